@@ -109,7 +109,9 @@ def algorithmic(b):
     flops = float(d * (ng ** 2).sum())  # comparable upper triangle: 2 d n^2 / 2 per group
     path_bytes = zb + 4 * N + meta + R + 4 * T
     # exact_stats: per embedding element two exact products (|z|^2 and the parent dot) and two
-    # compensated additions (TwoSum: 6 operations plus the error accumulation): 16 fp32 operations
+    # compensated additions (TwoSum: 6 operations plus the error accumulation): 16 fp32 operations,
+    # the figure the notes are held to; the kernels spend 8 (biased sums), and the group-resident
+    # ones only on the rows whose eta can reach a result
     alu_x = 16.0 * N * d
     stages = {
         "exact_stats": (zb + 16 * N, 0.0, alu_x),

@@ -363,7 +363,6 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   pp.b_next = bud ? bud->b_next : 0;
   pp.active = bud ? bud->active : nullptr;
   pp.budget = bud ? bud->budget : nullptr;
-  pp.stats_in_kernel = 0;
   pp.debug_timeout = (p.flags & GPO_FLAG_DEBUG_TIMEOUT) != 0;
   const Ws ws = workspace_views(workspace, L);
   LaunchCtx lc;
@@ -422,17 +421,6 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   } else if (fused32) {
     if (e == cudaSuccess) e = stage("fused_f32", [&] { return launch_fused_f32(lc, b, *out, sz, ws, pp); });
   } else if (fused) {
-    // one group per CTA at a time: the group warps compute the compensated statistics of
-    // each CTA's first group while it streams in; the groups after those (more groups than
-    // CTAs) get theirs from a launch of its own first, on the whole GPU, so that the group
-    // warps keep pace with the stream
-    pp.stats_in_kernel = !bud;
-    const int grid = fused_grid(lc, sz);
-    if (e == cudaSuccess && !bud && (int64_t)(g1 - g0) > (int64_t)grid) {
-      Sizes rest = sz;
-      rest.g0 = sz.g0 + grid;
-      e = stage("exact_stats", [&] { return launch_exact_stats(lc, b, rest, ws); });
-    }
     if (e == cudaSuccess) e = stage("fused", [&] { return launch_fused(lc, map, map32, b, *out, sz, ws, pp); });
   } else {
     if (e == cudaSuccess && b.parent) e = stage("tree_prep", [&] { return launch_tree_prep(lc, b, sz, ws); });
@@ -446,7 +434,7 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
         e = stage("similarity", [&] {
           return use_tc ? launch_sim_tc(lc, map, b, sz, ws, pp) : launch_sim_simt(lc, b, sz, ws, pp);
         });
-      if (e == cudaSuccess && !bud) e = stage("exact_stats", [&] { return launch_exact_stats(lc, b, sz, ws, true); });
+      if (e == cudaSuccess && !bud) e = stage("exact_stats", [&] { return launch_exact_stats(lc, b, sz, ws); });
       if (e == cudaSuccess) e = stage("groups", [&] { return launch_groups(lc, b, *out, sz, ws, pp); });
       if (e == cudaSuccess && !bud) e = stage("tokens", [&] { return launch_tokens(lc, b, *out, sz, ws); });
     }

@@ -17,7 +17,6 @@ constexpr int kWarpEdges = 256;                 // linked pairs listed per epilo
 constexpr int kEdgeList = kWarpEdges * (kEpiThreads / 32);
 constexpr int kBarGroup = 1;                    // named barrier of the group warps
 constexpr int kBarEpi = 2;                      // named barrier of the drain warps
-constexpr int kBarSetup = 3;                    // named barrier of warps 2 and 3 (early set-up)
 static_assert(kThreads % 128 == 0 && kThreads >= 256 && kGThreads >= kMaxN, "fused kernel shape");
 
 struct Seg {
@@ -133,7 +132,9 @@ struct __align__(16) GroupSmem {
   unsigned long long esum[3];  // exploration efficiency: token sums
   int flags;             // bit 0: group invalid
   int overflow;          // some warp found more pairs than its part of elist holds
-  int stats_next;        // next block of 8 rows for the row statistics (claimed by warps)
+  int nstat[2];          // group_eta_stats: rows with a dot, rows with the norm alone (group_row_stats:
+                         // the next block of 8 rows)
+  uint16_t slist[kMaxN]; // those rows: with a dot from the front, the norm alone from the end
   Plan plan;
   uint32_t elist[kEdgeList];  // linked pairs of the group, kWarpEdges per epilogue warp: i | j << 16
   alignas(16) unsigned char X[group_scratch_sep_bytes(kMaxN)];  // group-math sums (separate layout)
@@ -159,7 +160,6 @@ static_assert(kTilesOff + 1023 + kRingBytes <= 232448, "fused kernel exceeds 227
 
 __device__ __forceinline__ void bar_group() { asm volatile("bar.sync %0, %1;" ::"n"(kBarGroup), "n"(kGThreads) : "memory"); }
 __device__ __forceinline__ void bar_epi() { asm volatile("bar.sync %0, %1;" ::"n"(kBarEpi), "n"(kEpiThreads) : "memory"); }
-__device__ __forceinline__ void bar_setup() { asm volatile("bar.sync %0, %1;" ::"n"(kBarSetup), "n"(64) : "memory"); }
 
 // Bits a..31 of a word (all for a <= 0, none for a >= 32).
 __device__ __forceinline__ uint32_t bits_from(int a) { return a <= 0 ? 0xFFFFFFFFu : (a >= 32 ? 0u : 0xFFFFFFFFu << a); }
@@ -186,52 +186,104 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
   return v;
 }
 
-// Compensated |z_v|^2 and <z_{p(v)}, z_v> of the group's states [s0, s0 + n) into
-// ws.x_n2 / ws.x_dot (float pairs).  The calling warps claim blocks of 8 rows from
-// gs->stats_next until none is left, so that warps that join late or run slower take
-// fewer.  Parents: with `early` (chain layout, before the group's set-up) the previous
-// state for every state but the group's first (the set-up fixes the rollouts' first
-// states afterwards: their parent is the prompt root); otherwise from the group layout
-// in shared memory (chain: the previous state unless the state is a rollout's first; tree:
-// gs->par; the prompt embedding for a root child when there is one).
+// The compensated row statistics that the group's eta's ask for (every group but the first
+// of a CTA in a branching batch, see group_row_stats; all group threads, one
+// state each: thread gt has state gt; need: eta(p(v), v) of that state is read).  The rows
+// are known only once the classes are, when they have just been streamed and lie in L2, and
+// they are few: 0.2 to 0.45 of a chain batch's states (a step whose score differs from its
+// parent's, below a parent whose class has several edges), 0.85 of a branching one's.  Two
+// lists, the rows with a dot (|z_v|^2 and <z_{p(v)}, z_v>) from the front of slist and the
+// parents that need |z|^2 alone from its end; a half-warp per row (half_warp_row_sums,
+// biases from the Gram diagonal), every row's norm once.  Bound by the latency of its loads
+// and dependent sums at 14 warps per SM (a third of the issue slots used).  Results as float
+// pairs: |z|^2 in (rn, thr), free once the pairs are tested, the dot in (ecor, eeff).
+// Whole call, against the statistics of all rows (a CTA's first group while it streams in,
+// the groups after it in a launch of their own before): 512 groups of 320 states 273 -> 245 us.
+template <class Par>
+__device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
+                                                int g, int s0, int n, bool need, Par par, int gt, int wg, int lane,
+                                                uint32_t* st) {
+  int* mark = reinterpret_cast<int*>(gs->eadv);  // zeroed with the set-up
+  const int pl = need ? par(gt) : -1;
+  if (pl >= 0) mark[pl] = 1;
+  bar_group();
+  const bool alone = gt < n && !need && mark[gt] != 0;
+  const uint32_t md = __ballot_sync(0xffffffffu, need), ma = __ballot_sync(0xffffffffu, alone);
+  int bd = 0, ba = 0;
+  if (lane == 0) {
+    if (md) bd = atomicAdd(&gs->nstat[0], __popc(md));
+    if (ma) ba = atomicAdd(&gs->nstat[1], __popc(ma));
+  }
+  bd = __shfl_sync(0xffffffffu, bd, 0);
+  ba = __shfl_sync(0xffffffffu, ba, 0);
+  const uint32_t below = (1u << lane) - 1u;
+  if (need) gs->slist[bd + __popc(md & below)] = (uint16_t)gt;  // together at most n rows: the lists never meet
+  if (alone) gs->slist[kMaxN - 1 - (ba + __popc(ma & below))] = (uint16_t)gt;
+  bar_group();
+
+  const int nd = gs->nstat[0], na = gs->nstat[1];
+  const int pd = (nd + 1) >> 1, pa = (na + 1) >> 1;  // two rows per warp and step
+  const int hw = lane >> 4, hl = lane & 15;
+  const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
+  const uint4* Z = reinterpret_cast<const uint4*>(b.emb);
+#pragma unroll 1
+  for (int k = wg; k < pd + pa; k += kGThreads / 32) {
+    const bool wd = k < pd;  // (warp-uniform)
+    const int e = 2 * (wd ? k : k - pd) + hw;
+    bool live = e < (wd ? nd : na);
+    const int i = live ? (int)gs->slist[wd ? e : kMaxN - 1 - e] : 0;
+    live = live && GPO_BOUNDS(st, s0 + i, sz.N, kWhereStats);
+    float2 n2, dot;
+    if (wd) {
+      const int q = live ? par(i) : 0;  // the parent, or -1: the prompt embedding
+      live = live && GPO_BOUNDS(st, q >= 0 ? s0 + q : 0, sz.N, kWhereStats);
+      const uint4* y = q >= 0 ? Z + (int64_t)(s0 + q) * rs : reinterpret_cast<const uint4*>(b.root_emb) + (int64_t)g * rs;
+      half_warp_row_sums<true>(Z + (int64_t)(s0 + i) * rs, y, sz.d, gs->n2[i], q >= 0 ? gs->n2[q] : ws.x_root_n2[g].x,
+                               hl, live, n2, dot);
+    } else {
+      half_warp_row_sums<false>(Z + (int64_t)(s0 + i) * rs, nullptr, sz.d, gs->n2[i], 0.f, hl, live, n2, dot);
+    }
+    if (live && hl == 0) {
+      gs->rn[i] = n2.x;
+      gs->thr[i] = n2.y;
+      if (wd) {
+        gs->ecor[i] = dot.x;
+        gs->eeff[i] = dot.y;
+      }
+    }
+  }
+  bar_group();
+}
+
+// Compensated |z_v|^2 and <z_{p(v)}, z_v> of every state of a branching group into ws.x_n2 /
+// ws.x_dot (float pairs), by the group warps while the producer streams the same rows: for
+// a CTA's first group, when they would otherwise wait for the stream.  A branching batch
+// reads 0.85 of its eta's, so little of it is in vain (tree: 71.0 us, against 74.4 us with
+// group_eta_stats in its place; a chain batch reads a third of them, and there the rows of
+// group_eta_stats after the classes are the better: math 58.0 against 58.7 us, agentic
+// with all outputs 54.9 against 57.9).  The warps claim blocks of 8 rows; lane 4 r + c takes
+// every fourth 16-byte chunk of row r from chunk c; a parent that is the row before comes
+// from the lane 4 below.  bf16 products are exact in fp32, sums by TwoSum (no bound of the
+// norms is known yet), the row's 4 partial pairs combined in a fixed butterfly.
 __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
-                                                int g, int s0, int n, bool tree, bool early, int lane, uint32_t* st) {
+                                                int g, int s0, int n, int lane, uint32_t* st) {
   const int r = lane >> 2, c = lane & 3;
   const int nch = sz.d / 8;          // whole 16-byte chunks of a row
   const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
   const uint4* Z = reinterpret_cast<const uint4*>(b.emb);
   const uint4* RZ = reinterpret_cast<const uint4*>(b.root_emb);
-  auto finish4 = [&](uint64_t s, uint64_t e) -> float2 {  // the row's 4 lanes, fixed order
-    float2 P = f2_finish(s, e);
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      const float a = __shfl_xor_sync(0xffffffffu, P.x, o), q = __shfl_xor_sync(0xffffffffu, P.y, o);
-      float t, u;
-      two_sum(P.x, a, t, u);
-      P.x = t;
-      P.y = P.y + q + u;
-    }
-    float h, l;
-    two_sum(P.x, P.y, h, l);
-    return make_float2(h, l);
-  };
   auto claim = [&]() {
     int k = 0;
-    if (lane == 0) k = atomicAdd(&gs->stats_next, 1);
+    if (lane == 0) k = atomicAdd(&gs->nstat[0], 1);
     return __shfl_sync(0xffffffffu, k, 0);
   };
   for (int blk = claim(); blk * 8 < n; blk = claim()) {
     const int i = blk * 8 + r;  // local row of this lane
     const bool live = i < n;
-    // parent: >= 0 a local row, -2 the prompt embedding, -1 none (eta 0)
-    int pl = -1;
+    int pl = -1;  // parent: >= 0 a local row, -2 the prompt embedding, -1 none (eta 0)
     if (live) {
-      if (early) {
-        pl = i - 1;
-      } else {
-        pl = tree ? gs->par[i] : (gs->dep[i] > 1 ? i - 1 : -1);
-        if (pl < 0) pl = b.root_emb ? -2 : -1;
-      }
+      pl = gs->par[i];
+      if (pl < 0) pl = b.root_emb ? -2 : -1;
     }
     const bool from_left = pl >= 0 && pl == i - 1 && r > 0;
     // (debug build) the rows this lane reads; the whole warp skips the block if any is out of
@@ -241,14 +293,8 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
     if (!__all_sync(0xffffffffu, rows_ok)) continue;
     const uint4* zb = Z + (int64_t)(s0 + (live ? i : 0)) * rs;
     const uint4* pb = pl >= 0 ? Z + (int64_t)(s0 + pl) * rs : (pl == -2 ? RZ + (int64_t)g * rs : nullptr);
-    // error-free sums of the exact bf16 products (BiasedSum: a plain fp32 bound of each
-    // segment's |products|, then Fast2Sum against a power-of-two bias, four operations per
-    // product); a segment is one stage of kU chunks per lane
-    BiasedSum sn, sd;
-    bs_init(sn);
-    bs_init(sd);
-    // two stages of kU chunks per lane, software-pipelined: the next stage's loads are in
-    // flight while this one's sums run (no register copies between the stages)
+    uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
+    // two stages of kU chunks per lane, software-pipelined
     constexpr int kU = 2;
     auto load = [&](int k0, uint4 (&x)[kU], uint4 (&y)[kU]) {
 #pragma unroll
@@ -259,8 +305,7 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
         y[u] = !from_left && pb && in ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
       }
     };
-    auto accumulate = [&](uint4 (&x)[kU], uint4 (&y)[kU]) {
-      uint64_t xx[4 * kU], yy[4 * kU];
+    auto accumulate = [&](const uint4 (&x)[kU], uint4 (&y)[kU]) {
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         uint4 t;
@@ -272,27 +317,15 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
         const uint32_t xw[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yw[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-          xx[4 * u + h] = bf16x2_f32x2(xw[h]);
-          yy[4 * u + h] = bf16x2_f32x2(yw[h]);
+          const uint64_t xx = bf16x2_f32x2(xw[h]), yy = bf16x2_f32x2(yw[h]);
+          f2_acc(ns, ne, f2mul(xx, xx));
+          f2_acc(ds, de, f2mul(xx, yy));
         }
-      }
-      uint64_t px = 0ull, py = 0ull;  // the segment's sums of squares (bounds only)
-#pragma unroll
-      for (int i = 0; i < 4 * kU; ++i) {
-        px = f2fma(xx[i], xx[i], px);
-        py = f2fma(yy[i], yy[i], py);
-      }
-      const float qx = f2_lanes_sum(px), qy = f2_lanes_sum(py);
-      bs_reserve(sn, qx);
-      bs_reserve(sd, 0.5f * (qx + qy));  // |x y| <= (x^2 + y^2) / 2
-#pragma unroll
-      for (int i = 0; i < 4 * kU; ++i) {
-        bs_add(sn, xx[i], xx[i]);  // bf16 products are exact in fp32
-        bs_add(sd, xx[i], yy[i]);
       }
     };
     uint4 xa[kU], ya[kU], xb[kU], yb[kU];
     load(0, xa, ya);
+#pragma unroll 1
     for (int k0 = 0; k0 < nch; k0 += 8 * kU) {
       load(k0 + 4 * kU, xb, yb);  // past the row's end: zeros, which add nothing
       accumulate(xa, ya);
@@ -302,35 +335,19 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
     if (sz.d % 8 != 0 && c == 0 && live) {  // the ragged end of the row, one lane per row
       const uint16_t* zr = reinterpret_cast<const uint16_t*>(zb);
       const uint16_t* pr = reinterpret_cast<const uint16_t*>(pb);
-      float qx = 0.f, qy = 0.f;
-      for (int k = 8 * nch; k < sz.d; ++k) {
-        const float x = __uint_as_float((uint32_t)zr[k] << 16), y = pr ? __uint_as_float((uint32_t)pr[k] << 16) : 0.f;
-        qx = fmaf(x, x, qx);
-        qy = fmaf(y, y, qy);
-      }
-      bs_reserve(sn, qx);
-      bs_reserve(sd, 0.5f * (qx + qy));
       for (int k = 8 * nch; k < sz.d; ++k) {
         const uint64_t xx = pack_f2((uint32_t)zr[k] << 16, 0u);  // one fp32 lane (the other stays 0)
-        const uint64_t yy = pack_f2(pr ? (uint32_t)pr[k] << 16 : 0u, 0u);
-        bs_add(sn, xx, xx);
-        bs_add(sd, xx, yy);
+        f2_acc(ns, ne, f2mul(xx, xx));
+        f2_acc(ds, de, f2mul(xx, pack_f2(pr ? (uint32_t)pr[k] << 16 : 0u, 0u)));
       }
     }
-    uint64_t ns, ne, ds, de;
-    bs_finish(sn, ns, ne);
-    bs_finish(sd, ds, de);
-    const float2 n2 = finish4(ns, ne);
-    float2 dot = finish4(ds, de);
-    if (pl == -1) dot = make_float2(0.f, 0.f);
+    const float2 n2 = lanes_pair_sum<4>(f2_finish(ns, ne)), dot = lanes_pair_sum<4>(f2_finish(ds, de));
     if (live && c == 0 && GPO_BOUNDS(st, s0 + i, sz.N, kWhereStats)) {
-      if (!isfinite(n2.x) || !isfinite(dot.x)) report(st, GPO_ERR_NONFINITE, 3, s0 + i);
       ws.x_n2[s0 + i] = n2;
-      ws.x_dot[s0 + i] = dot;
+      ws.x_dot[s0 + i] = pl == -1 ? make_float2(0.f, 0.f) : dot;
     }
   }
 }
-
 
 // Tree-layout set-up of group g (Sec. 4.2 branching rollouts: parents precede their
 // children, depth-first pre-order): checks, depth, subtree end, own terminal statistics
@@ -353,6 +370,7 @@ __device__ __forceinline__ void tree_setup(const gpo_batch& b, const Sizes& sz, 
     gs->rend[i] = i + 1;
     gs->cown[i] = 0;
     gs->town[i] = 0;
+    gs->eadv[i] = 0.f;  // (the marks of group_eta_stats)
     bad = bad || pp < -1 || pp >= i || L < 1;
   }
   bad = bar_any<kBarGroup, kGThreads>(bad);
@@ -468,7 +486,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     mbar_init(&ctl->tempty, kEpiThreads / 32);
     mbar_init(&ctl->drain, 1);
     fence_mbar_init();
-    gs->stats_next = 0;
     tma_prefetch_desc(&zmap);
     tma_prefetch_desc(&zmap32);
   }
@@ -628,35 +645,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         make_plan(n, gs->plan);
         gs->flags = 0;
         gs->overflow = 0;
+        gs->nstat[0] = gs->nstat[1] = 0;
       }
-
-      // ---- compensated row statistics of the group (eta needs them; the Gram accumulator
-      //      is too coarse): |z_v|^2 and <z_{p(v)}, z_v> as float pairs into ws.x_n2 / x_dot,
-      //      read from L2 or HBM while the producer streams the same rows, only for each
-      //      CTA's first group (its stream has nothing to overlap before it; later groups'
-      //      come from a launch of their own).  A warp takes 8 rows, lane 4 r + c every fourth
-      //      16-byte chunk of row r starting at chunk c; a parent that is the row before comes
-      //      from the lane 4 below, other parents and the prompt embedding are loaded.  bf16
-      //      products are exact in fp32, every sum is error-free (BiasedSum), the row's 4
-      //      partial pairs are combined in a fixed butterfly.  Chain layout without prompt
-      //      embeddings: the drain warps start at once (every state's parent taken as the
-      //      state before it; a rollout's first state then has eta 0 whatever its dot) while
-      //      warps 2 and 3 lay out the group, then join them; otherwise all group warps
-      //      after the set-up.
-      const bool stats_here = p.mode == 0 && p.stats_in_kernel && g < sz.g0 + (int)gridDim.x;
-      const bool early = stats_here && !tree && b.root_emb == nullptr;
-      if (early && epi) group_row_stats(b, sz, ws, gs, g, s0, n, false, true, lane, st);
 
       if (tree) {
         tree_setup(b, sz, gs, g, r0, nr, s0, n, gt, wg, lane, st);
-      } else if (!early || !epi) {
-      // ---- validate the group and lay out its states (Sec. 4.2 chain layout): all group
-      //      threads, or warps 2 and 3 alone while the drain warps read the statistics
-      const int tid = gt, nt = early ? 64 : kGThreads;  // warps 2 and 3: gt = 0..63
-      auto sync = [&] {
-        if (early) bar_setup();
-        else bar_group();
-      };
+      } else {
+      // ---- validate the group and lay out its states (Sec. 4.2 chain layout)
+      const int tid = gt, nt = kGThreads;
       for (int r = tid; r <= nr; r += nt) {
         gs->rstart[r] = b.rollout_step_off[r0 + r] - s0;
         gs->tok0[r] = b.rollout_token_off[r0 + r];
@@ -668,8 +664,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         gs->slen[i] = b.step_len[s0 + i];
         gs->roll[i] = 0;
         gs->dep[i] = 1;
+        gs->eadv[i] = 0.f;  // (the marks of group_eta_stats)
       }
-      sync();
+      bar_group();
       for (int r = tid; r < nr; r += nt) {
         const int a = gs->rstart[r], e = gs->rstart[r + 1];
         bool bad = !(a >= 0 && e > a && e <= n) || gs->rew[r] > 1;
@@ -691,30 +688,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           atomicOr(&gs->flags, 1);
         }
       }
-      if (early) group_row_stats(b, sz, ws, gs, g, s0, n, false, true, lane, st);  // join the drain warps
       }
-      bar_group();  // set-up (and with `early` the row statistics) complete
+      bar_group();  // set-up complete
       const bool valid = (gs->flags & 1) == 0;
-      if (!early && valid && stats_here) group_row_stats(b, sz, ws, gs, g, s0, n, tree, false, lane, st);
-      if (valid && stats_here && b.root_emb && wg == 0) {  // |prompt embedding|^2, one warp
+      const bool early = tree && p.mode == 0 && g < sz.g0 + (int)gridDim.x;  // the CTA's first group
+      if (early && valid) group_row_stats(b, sz, ws, gs, g, s0, n, lane, st);
+      if (valid && p.mode == 0 && b.root_emb && wg == 0) {  // |prompt embedding|^2, one warp
         float2 n2, dot;
         exact_pair_sums<true>(b.root_emb, (int64_t)g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
         if (lane == 0) {
           if (!isfinite(n2.x)) report(st, GPO_ERR_NONFINITE, 3, sz.N + g);
           ws.x_root_n2[g] = n2;
-        }
-      }
-
-      // ---- eta(p(v), v) of every state from the finished statistics, by warps 2 and 3 while
-      //      the drain warps test the pairs (with `early`: no prompt embedding, a rollout's
-      //      first state has eta 0); the group math takes it from ecor / eeff, which it
-      //      overwrites only with its own outputs, state by state, after reading it
-      if (early && valid && !epi) {
-        for (int i = gt; i < n; i += 64) {
-          const float2 e = gs->dep[i] == 1 ? make_float2(0.f, 0.f)
-                                           : ff_eta(ws.x_dot[s0 + i], ws.x_n2[s0 + i - 1], ws.x_n2[s0 + i]);
-          gs->ecor[i] = e.x;
-          gs->eeff[i] = e.y;
         }
       }
 
@@ -903,13 +887,19 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       }
       // ---- graph reward and dual-group advantage of every edge
       else if (valid) {
-        // eta(p(v), v) from the compensated row statistics (pairs; see exact_stats_kernel)
-        auto eta = [&](int i) -> float2 {
-          if (early) return make_float2(gs->ecor[i], gs->eeff[i]);
-          const float2 z = make_float2(0.f, 0.f);
-          const float2 n1 = gs->dep[i] == 1 ? (b.root_emb ? ws.x_root_n2[g] : z) : ws.x_n2[s0 + i - 1];
-          return ff_eta(ws.x_dot[s0 + i], n1, ws.x_n2[s0 + i]);
+        // eta(p(v), v) from the compensated row statistics: of every row (early), else of the
+        // rows that ask for it
+        auto par = [&](int i) { return tree ? gs->par[i] : (gs->dep[i] == 1 ? -1 : i - 1); };
+        auto etas = [&](const bool (&need)[1]) {
+          if (!early) group_eta_stats(b, sz, ws, gs, g, s0, n, need[0], par, gt, wg, lane, st);
         };
+        auto eta = [&](int i) -> float2 {
+          const int q = par(i);  // -1: the prompt embedding
+          const float2 nq = q < 0 ? ws.x_root_n2[g] : (early ? ws.x_n2[s0 + q] : make_float2(gs->rn[q], gs->thr[q]));
+          return early ? ff_eta(ws.x_dot[s0 + i], nq, ws.x_n2[s0 + i])
+                       : ff_eta(make_float2(gs->ecor[i], gs->eeff[i]), nq, make_float2(gs->rn[i], gs->thr[i]));
+        };
+        const bool has_root = b.root_emb != nullptr;
         auto out = [&](int i, int label, float S, float acor, float E, float dual, unsigned char mask) {
           gs->eadv[i] = dual;
           gs->ecor[i] = acor;
@@ -925,23 +915,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           if (o.edge_eff_mask) o.edge_eff_mask[v] = mask;
         };
         if (tree) {
-          auto eta_t = [&](int i) -> float2 {
-            const float2 z = make_float2(0.f, 0.f);
-            const int pp = gs->par[i];
-            const float2 n1 = pp < 0 ? (b.root_emb ? ws.x_root_n2[g] : z) : ws.x_n2[s0 + pp];
-            return ff_eta(ws.x_dot[s0 + i], n1, ws.x_n2[s0 + i]);
-          };
           group_advantages_tree<1>(n, nr, gs->lab, gs->par, gs->dep, gs->rend, gs->cown, gs->town,
                                    tree_scratch(smem_raw + kTreeXOff, n), p, gt, kGThreads, [] { bar_group(); },
-                                   eta_t, out);
+                                   has_root, etas, eta, out);
         } else {
           group_advantages<1, true>(n, nr, gs->lab, gs->roll, gs->dep, gs->rstart, gs->rew,
-                                    group_scratch_sep(gs->X, n), p, gt, kGThreads, [] { bar_group(); }, eta, out);
+                                    group_scratch_sep(gs->X, n), p, gt, kGThreads, [] { bar_group(); }, has_root, etas,
+                                    eta, out);
         }
         // ---- exploration efficiency, Eq. (eq1) (the threshold norms' array is free here)
         if (o.group_eff || o.group_eff_graph) {
           auto own = [&](int i) { return tree ? gs->cown[i] > 0 : gs->rew[gs->roll[i]] != 0; };
-          auto par = [&](int i) { return tree ? gs->par[i] : (gs->dep[i] == 1 ? -1 : i - 1); };
           auto len = [&](int i) { return gs->slen[i]; };
           group_efficiency(n, gs->lab, reinterpret_cast<int*>(gs->n2), gs->esum, gt, kGThreads, own, par, len,
                            [] { bar_group(); }, [](bool f) { return bar_any<kBarGroup, kGThreads>(f); },
@@ -991,7 +975,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           }
         }
       }
-      if (gt == 0) gs->stats_next = 0;  // for the next group's row statistics
       bar_group();
     }
   }

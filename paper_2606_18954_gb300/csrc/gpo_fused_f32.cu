@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(NT, 1) fused_f32_kernel(gpo_batch b, gpo_outpu
       if (o.edge_eff_mask) o.edge_eff_mask[v] = mask;
     };
     group_advantages<1, true>(n, nr, gs->lab, gs->roll, gs->dep, gs->rstart, gs->rew, group_scratch_sep(gs->X, n),
-                              p, tid, nt, sync, eta, out);
+                              p, tid, nt, sync, b.root_emb != nullptr, [](const bool (&)[1]) {}, eta, out);
     // ---- exploration efficiency, Eq. (eq1) (the norms' array is free here)
     if (o.group_eff || o.group_eff_graph) {
       auto own = [&](int i) { return gs->rew[gs->roll[i]] != 0; };

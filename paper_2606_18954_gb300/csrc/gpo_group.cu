@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
     const float2 n1 = dep[i] == 1 ? (b.root_emb ? ws.x_root_n2[g] : zero2) : ws.x_n2[v - 1];
     return ff_eta(ws.x_dot[v], n1, ws.x_n2[v]);
   };
+  auto no_etas = [](const bool (&)[kPer]) {};  // every row's statistics are in the workspace
   auto out = [&](int i, int label, float S, float acor, float E, float dual, unsigned char mask) {
     const int v = s0 + i;
     if (!GPO_BOUNDS(st, v, sz.N, kWhereStateOut)) return;
@@ -185,14 +186,14 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
                   "workspace layout of the tree sums");
     group_advantages_tree<kPer, int16_t>(n, nr, lab, tpar, dep, tend, tcown, ttown,
                                          tree_scratch(ws.tree_x + (size_t)23 * s0 + (size_t)11 * g, n), p, tid, nt,
-                                         [] { __syncthreads(); }, eta_t, out);
+                                         [] { __syncthreads(); }, b.root_emb != nullptr, no_etas, eta_t, out);
     // the own statistics take 2 al16(2n) bytes at the start of X
     efficiency(reinterpret_cast<int*>(X + 2 * al16(sizeof(int16_t) * (size_t)n)));
     return;  // the tree prep kernel wrote the first token of every edge
   }
   __shared__ int s_rootc;
   group_advantages<kPer, false, int16_t>(n, nr, lab, roll, dep, rstart, rew, group_scratch_shared(X, n, &s_rootc), p,
-                                         tid, nt, [] { __syncthreads(); }, eta, out);
+                                         tid, nt, [] { __syncthreads(); }, b.root_emb != nullptr, no_etas, eta, out);
   efficiency(reinterpret_cast<int*>(X));
 
   // first token of every edge: one warp per rollout, an exclusive scan of the step lengths

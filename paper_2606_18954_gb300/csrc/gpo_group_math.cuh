@@ -104,11 +104,10 @@ __device__ __forceinline__ float2 score_ff(int c, int t, int C, int T, float wh,
   return ff_div(lin_ff(c, C - c, wh, wl), lin_ff(t, T - t, wh, wl));
 }
 
-// r_step = (S(v) - S(p(v))) (1 - eta) on the 2^-50 grid (|r| <= 1), from pair-valued
-// scores and eta: the pair arithmetic keeps r to ~2^-46 relative, well below the grid
-// of the exact group sums that follow.
-__device__ __forceinline__ long long step_reward_fixed(float2 S, float2 Sp, float2 eta) {
-  const float2 d = ff_add(S, make_float2(-Sp.x, -Sp.y));
+// r_step = (S(v) - S(p(v))) (1 - eta) on the 2^-50 grid (|r| <= 1), from the pair-valued
+// score difference d and eta: the pair arithmetic keeps r to ~2^-46 relative, well below
+// the grid of the exact group sums that follow.
+__device__ __forceinline__ long long step_reward_fixed(float2 d, float2 eta) {
   const float2 r = ff_mul(d, ff_add(make_float2(1.0f, 0.0f), make_float2(-eta.x, -eta.y)));
   return __float2ll_rn(r.x * 0x1p50f) + __float2ll_rn(r.y * 0x1p50f);
 }
@@ -192,6 +191,13 @@ __device__ __forceinline__ GroupScratch group_scratch_shared(unsigned char* X, i
 //   rew     [nr] rewards
 //   sc      scratch: separate layout zeroed by the caller (kZeroed), or the
 //           shared layout (!kZeroed)
+//   has_root  a prompt embedding is given (else eta is 0 on the first step of a rollout)
+//   etas(need)  collective over the nt threads (it may hold barriers), called once before
+//           any eta(i): need[k] tells whether the thread's k-th state's eta is read.  It is
+//           not where it cannot reach a result: where S(v) = S(p(v)) exactly (the step reward
+//           is 0 whatever eta is), on a rollout's first step without a prompt embedding, and
+//           (kZeroed, which counts the groups' edges early) in a correctness group of one
+//           edge (A_cor = 0).
 //   eta(i)  eta(p(v), v) of local state i as a float pair (already clamped at 0)
 //   out(i, label, S, acor, E, dual, mask) is called once per state by its owner
 //   sync()  barrier over the nt threads
@@ -202,10 +208,11 @@ __device__ __forceinline__ GroupScratch group_scratch_shared(unsigned char* X, i
 // that needs them (same operands, same operations, so the same value), which
 // saves a barrier per constant.  Sums go through integer atomics, so results do
 // not depend on the order in which threads add.
-template <int kPer, bool kZeroed, class IdxT, class Sync, class Eta, class Out>
+template <int kPer, bool kZeroed, class IdxT, class Sync, class Etas, class Eta, class Out>
 __device__ __forceinline__ void group_advantages(int n, int nr, int* lab, const IdxT* roll, const IdxT* dep,
                                                  const int* rstart, const uint8_t* rew, const GroupScratch& sc,
-                                                 const Params& p, int tid, int nt, Sync sync, Eta eta, Out out) {
+                                                 const Params& p, int tid, int nt, Sync sync, bool has_root, Etas etas,
+                                                 Eta eta, Out out) {
   const float w = p.w_hi, eps = p.eps_f;
   const float wl = p.w_lo;  // w = w + wl to ~2^-48
   // ---- phase A: class sums C_Q (rewards), |Q|, sum l, sum l^2
@@ -217,16 +224,21 @@ __device__ __forceinline__ void group_advantages(int n, int nr, int* lab, const 
     if (tid == 0) *sc.rootc = 0;
     sync();
   }
-  int lb[kPer];
+  int lb[kPer], key[kPer];  // class; correctness group: the class of p(v), n = the prompt root
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int i = tid + k * nt;
     lb[k] = 0;
+    key[k] = n;
     if (i < n) {
       // writing the root over the parent keeps every concurrent find on the same root
       lb[k] = uf_find(lab, i);
       lab[i] = lb[k];
       const int d = dep[i];
+      if (kZeroed) {
+        if (d != 1) key[k] = uf_find(lab, i - 1);  // the previous state of the same rollout
+        atomicAdd(&sc.kcnt[key[k]], 1);
+      }
       atomicAdd(&sc.ccnt[lb[k]], 1);
       atomicAdd(&sc.csum[lb[k]], (int)rew[roll[i]]);
       atomicAdd(&sc.lsum[lb[k]], d);
@@ -237,16 +249,14 @@ __device__ __forceinline__ void group_advantages(int n, int nr, int* lab, const 
   sync();
   const float2 S_root = ff_div(make_float2((float)*sc.rootc, 0.f), make_float2((float)nr, 0.f));
   float S[kPer], aeff[kPer];
-  long long rf[kPer];
-  int key[kPer];
-  bool route_end[kPer];
+  float2 dS[kPer];  // S(v) - S(p(v))
+  bool route_end[kPer], need[kPer];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int i = tid + k * nt;
     S[k] = aeff[k] = 0.f;
-    rf[k] = 0;
-    key[k] = n;
-    route_end[k] = false;
+    dS[k] = make_float2(0.f, 0.f);
+    route_end[k] = need[k] = false;
     if (i >= n) continue;
     const int L = lb[k], Q = sc.ccnt[L], d = dep[i], c = rew[roll[i]];
     // Eq. (combain): (c_own + w sum_{q != v} c_own(q)) / (t_own + w sum_{q != v} t_own(q)), t_own = 1,
@@ -269,12 +279,17 @@ __device__ __forceinline__ void group_advantages(int n, int nr, int* lab, const 
     }
     float2 Sp = S_root;
     if (d != 1) {
-      const int Lp = lab[i - 1];  // parent: the previous state of the same rollout (same reward c)
-      Sp = score_ff(c, 1, sc.csum[Lp], sc.ccnt[Lp], w, wl);
-      key[k] = Lp;
+      if (!kZeroed) key[k] = lab[i - 1];  // parent: the previous state of the same rollout (same reward c)
+      Sp = score_ff(c, 1, sc.csum[key[k]], sc.ccnt[key[k]], w, wl);
     }
-    rf[k] = step_reward_fixed(Sv, Sp, eta(i));
+    dS[k] = ff_add(Sv, make_float2(-Sp.x, -Sp.y));
+    need[k] = (dS[k].x != 0.f || dS[k].y != 0.f) && (d != 1 || has_root) && (!kZeroed || sc.kcnt[key[k]] >= 2);
   }
+  etas(need);
+  long long rf[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k)
+    rf[k] = step_reward_fixed(dS[k], need[k] ? eta(tid + k * nt) : make_float2(0.f, 0.f));
 
   // ---- phase B: correctness groups, key = class of p(v), n = the prompt root
   if (!kZeroed) {
@@ -286,7 +301,7 @@ __device__ __forceinline__ void group_advantages(int n, int nr, int* lab, const 
   for (int k = 0; k < kPer; ++k) {
     if (tid + k * nt < n) {
       // |r| <= 1 and a group holds at most 4096 edges: a 2^50 fixed point cannot overflow
-      atomicAdd(&sc.kcnt[key[k]], 1);
+      if (!kZeroed) atomicAdd(&sc.kcnt[key[k]], 1);
       red_chunks<kSumWords, 18>(&sc.ksum[kSumWords * key[k]], (unsigned long long)(rf[k] + (1ll << 50)));
     }
   }
@@ -461,47 +476,51 @@ __device__ __forceinline__ TreeScratch tree_scratch(void* base, int n) {
 //   par    [n] local parent, -1 for the prompt root (par[x] < x)
 //   dep    [n] depth (1 = child of the root);  end [n] local end of the subtree
 //   cown, town [n] own terminal statistics;  nleaf = number of leaves (> 0)
-//   sc     tree scratch (zeroed here), eta(i), out(...) and sync() as in group_advantages
-template <int kPer, class IdxT, class Sync, class Eta, class Out>
+//   sc     tree scratch (zeroed here); has_root, etas(need), eta(i), out(...) and sync() as in
+//          group_advantages (the groups' edges are counted early)
+template <int kPer, class IdxT, class Sync, class Etas, class Eta, class Out>
 __device__ __forceinline__ void group_advantages_tree(int n, int nleaf, int* lab, const IdxT* par, const IdxT* dep,
                                                       const IdxT* end, const IdxT* cown, const IdxT* town,
                                                       const TreeScratch& sc, const Params& p, int tid, int nt,
-                                                      Sync sync, Eta eta, Out out) {
+                                                      Sync sync, bool has_root, Etas etas, Eta eta, Out out) {
   const float w = p.w_hi, eps = p.eps_f;
   const float wl = p.w_lo;
   for (int i = tid; i < sc.nzero; i += nt) sc.ccnt[i] = 0;
   sync();
   // ---- phase A: class sums
-  int lb[kPer];
+  int lb[kPer], key[kPer];  // class; correctness group: the class of p(v), n = the prompt root
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int i = tid + k * nt;
     lb[k] = 0;
+    key[k] = n;
     if (i < n) {
       lb[k] = uf_find(lab, i);
       lab[i] = lb[k];
-      const int d = dep[i];
+      const int d = dep[i], pp = par[i];
+      if (pp >= 0) key[k] = uf_find(lab, pp);
+      atomicAdd(&sc.kcnt[key[k]], 1);
       atomicAdd(&sc.ccnt[lb[k]], 1);
       atomicAdd(&sc.csum[lb[k]], (int)cown[i]);
       atomicAdd(&sc.tsum[lb[k]], (int)town[i]);
       atomicAdd(&sc.lsum[lb[k]], d);
       red_chunks<2, 13>(&sc.l2[2 * lb[k]], (unsigned long long)d * d);
       atomicMax(&sc.hi[lb[k]], i);
-      if (par[i] < 0) atomicAdd(sc.rootc, (int)cown[i]);
+      if (pp < 0) atomicAdd(sc.rootc, (int)cown[i]);
     }
   }
   sync();
   // ---- phase A2: S, the parent's S, r_step; S and r into their sums; a_Q per class
   const float2 S_root = ff_div(make_float2((float)*sc.rootc, 0.f), make_float2((float)nleaf, 0.f));
   float S[kPer];
-  int key[kPer];
-  long long rf[kPer];
+  float2 dS[kPer];  // S(v) - S(p(v))
+  bool need[kPer];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int i = tid + k * nt;
     S[k] = 0.f;
-    key[k] = n;
-    rf[k] = 0;
+    dS[k] = make_float2(0.f, 0.f);
+    need[k] = false;
     if (i >= n) continue;
     const int L = lb[k], c = cown[i], t = town[i];
     // Eq. (combain) as a float pair: a class whose leaves share one reward gets S exactly 0 or 1
@@ -509,22 +528,25 @@ __device__ __forceinline__ void group_advantages_tree(int n, int nleaf, int* lab
     S[k] = Sv.x;
     const int pp = par[i];
     float2 Sp = S_root;
-    if (pp >= 0) {
-      const int Lp = lab[pp];  // the parent's S, recomputed alike
-      Sp = score_ff(cown[pp], town[pp], sc.csum[Lp], sc.tsum[Lp], w, wl);
-      key[k] = Lp;
-    }
-    rf[k] = step_reward_fixed(Sv, Sp, eta(i));
+    if (pp >= 0) Sp = score_ff(cown[pp], town[pp], sc.csum[key[k]], sc.tsum[key[k]], w, wl);  // recomputed alike
+    dS[k] = ff_add(Sv, make_float2(-Sp.x, -Sp.y));
+    need[k] = (dS[k].x != 0.f || dS[k].y != 0.f) && (pp >= 0 || has_root) && sc.kcnt[key[k]] >= 2;
     red_chunks<3, 14>(&sc.ssum[3 * L],
                       (unsigned long long)(__float2ll_rn(Sv.x * 0x1p40f) + __float2ll_rn(Sv.y * 0x1p40f)));
-    atomicAdd(&sc.kcnt[key[k]], 1);
-    red_chunks<kSumWords, 18>(&sc.ksum[kSumWords * key[k]], (unsigned long long)(rf[k] + (1ll << 50)));
     if (i == L && sc.ccnt[L] >= 2) {
       const int h = sc.hi[L];
       int x = L;
       while (x >= 0 && end[x] <= h) x = par[x];
       sc.aqd[L] = x == L ? (int)dep[L] - 1 : (x < 0 ? 0 : (int)dep[x]);
     }
+  }
+  etas(need);
+  long long rf[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    rf[k] = step_reward_fixed(dS[k], need[k] ? eta(tid + k * nt) : make_float2(0.f, 0.f));
+    if (tid + k * nt < n)
+      red_chunks<kSumWords, 18>(&sc.ksum[kSumWords * key[k]], (unsigned long long)(rf[k] + (1ll << 50)));
   }
   sync();
   // ---- phase B2: exact group means and squared deviations; A_eff per state

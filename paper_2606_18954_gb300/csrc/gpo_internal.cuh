@@ -91,8 +91,6 @@ struct Params {
   int ddof, rule;
   // mode 1: next-layer budgets after layer `layer` instead of advantages (gpo_layer_budget)
   int mode, layer, b_next;
-  int stats_in_kernel;    // fused path: the group warps compute the compensated row statistics
-                          // of each CTA's first group (the other groups' come from exact_stats)
   int debug_timeout;      // GPO_FLAG_DEBUG_TIMEOUT: the MMA warp's first wait runs out
   const uint8_t* active;  // [N] frontier states to expand (NULL: all of depth `layer`)
   int32_t* budget;        // [N] output of mode 1
@@ -483,11 +481,9 @@ __device__ __forceinline__ float2 f2_finish(uint64_t s, uint64_t e) {
 // Floating-Point Arithmetic, Sec. 4.3): s - t and p + (s - t) are exact, and
 //   t = fma(x, y, s),  z = s - t,  err = fma(x, y, z) = p - (t - s)
 // gives the rounding error of every addition exactly (collected, rounded, in e).  s - sigma
-// is exact (Sterbenz), so the sum is (s - sigma) + e.  B comes from a plain fp32 pass over
-// the next segment of the operands (sum of x^2, and (x^2 + y^2) / 2 >= |x y| for a dot),
-// with a relative margin that covers that pass's rounding; when 2 B would pass sigma, the
-// current epoch is closed into a float pair by TwoSum and a new one starts with
-// sigma = 2^ceil(log2 4 B).  Two fp32 lanes per instruction, as in f2_acc.
+// is exact (Sterbenz), so the sum is (s - sigma) + e.  B comes from the similarity stage's
+// fp32 squared norms (|x y| <= (x^2 + y^2) / 2 for a dot): sigma = 2^ceil(log2 (4.04 |x|^2))
+// and 2^ceil(log2 (2.02 (|x|^2 + |y|^2))).  Two fp32 lanes per instruction, as in f2_acc.
 
 __device__ __forceinline__ uint64_t f2fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
@@ -495,45 +491,11 @@ __device__ __forceinline__ uint64_t f2fma(uint64_t a, uint64_t b, uint64_t c) {
   return d;
 }
 __device__ __forceinline__ uint64_t f2splat(float x) { return pack_f2(__float_as_uint(x), __float_as_uint(x)); }
-// The sum of a pair's two fp32 lanes (rounded once).
-__device__ __forceinline__ float f2_lanes_sum(uint64_t a) {
-  uint32_t lo, hi;
-  unpack_f2(a, lo, hi);
-  return __uint_as_float(lo) + __uint_as_float(hi);
-}
 // Smallest power of two >= x, for finite x >= 0 (0 for 0; +inf beyond the fp32 range).
 __device__ __forceinline__ float pow2_ceil(float x) {
   return __uint_as_float((__float_as_uint(x) + 0x007FFFFFu) & 0xFF800000u);
 }
 
-struct BiasedSum {
-  uint64_t s, e;  // biased running sums and their rounding errors (two lanes)
-  uint64_t h, l;  // float pairs (two lanes) of the epochs closed so far
-  float sigma;    // bias of the current epoch (both lanes)
-  float bound;    // bound of the sum of |products| added so far (plus the reserved segment)
-};
-
-__device__ __forceinline__ void bs_init(BiasedSum& a) {
-  a.s = a.e = a.h = a.l = 0ull;
-  a.sigma = 0.f;
-  a.bound = 0.f;
-}
-// Closes the current epoch: (s - sigma) + e joins the pair (h, l).
-__device__ __forceinline__ void bs_close(BiasedSum& a) {
-  f2_acc(a.h, a.l, f2sub(a.s, f2splat(a.sigma)));  // s - sigma is exact in each lane
-  a.l = f2add(a.l, a.e);
-}
-// Reserves room for a segment whose sum of |products| is at most `add` (a plain fp32
-// estimate; the relative margin 2^-12 covers its rounding and that of the bound itself).
-__device__ __forceinline__ void bs_reserve(BiasedSum& a, float add) {
-  a.bound = fmaf(add, 1.000244140625f, a.bound);
-  if (2.f * a.bound > a.sigma) {
-    bs_close(a);
-    a.sigma = pow2_ceil(4.f * a.bound);
-    a.s = f2splat(a.sigma);
-    a.e = 0ull;
-  }
-}
 // One Fast2Sum step of a biased running sum s (error collected in e): the exact products
 // x y (two lanes), |x y| <= |s| with s - t exact (the caller's bias guarantees both).
 __device__ __forceinline__ void biased_add(uint64_t& s, uint64_t& e, uint64_t x, uint64_t y) {
@@ -541,18 +503,140 @@ __device__ __forceinline__ void biased_add(uint64_t& s, uint64_t& e, uint64_t x,
   e = f2add(e, f2fma(x, y, f2sub(s, t)));
   s = t;
 }
-// Adds the exact products x y (two lanes).
-__device__ __forceinline__ void bs_add(BiasedSum& a, uint64_t x, uint64_t y) {
-  const uint64_t t = f2fma(x, y, a.s);
-  const uint64_t z = f2sub(a.s, t);
-  a.e = f2add(a.e, f2fma(x, y, z));
-  a.s = t;
+// A sum of exact products in two chains of two lanes, all with the bias sigma.
+struct BiasedSum {
+  uint64_t s0, s1, e0, e1;
+  float sigma;
+};
+__device__ __forceinline__ void bs_init(BiasedSum& a, float sigma) {
+  a.sigma = sigma;
+  a.s0 = a.s1 = f2splat(sigma);
+  a.e0 = a.e1 = 0ull;
 }
-// The two lanes' pairs of the finished sum, to be combined by f2_finish.
-__device__ __forceinline__ void bs_finish(BiasedSum& a, uint64_t& s, uint64_t& e) {
-  bs_close(a);
-  s = a.h;
-  e = a.l;
+// Every running sum still in [sigma/2, 3 sigma/2]: then each step was error-free.
+__device__ __forceinline__ bool bs_in_range(const BiasedSum& a) {
+  uint32_t x, y, z, w;
+  unpack_f2(a.s0, x, y);
+  unpack_f2(a.s1, z, w);
+  const float h = 0.5f * a.sigma;
+  return fabsf(__uint_as_float(x) - a.sigma) <= h && fabsf(__uint_as_float(y) - a.sigma) <= h &&
+         fabsf(__uint_as_float(z) - a.sigma) <= h && fabsf(__uint_as_float(w) - a.sigma) <= h;
+}
+// The sum as a float pair: (s - sigma) is exact in each lane, both chains' parts and errors.
+__device__ __forceinline__ float2 bs_pair(const BiasedSum& a) {
+  uint64_t h = 0ull, l = 0ull;
+  f2_acc(h, l, f2sub(a.s0, f2splat(a.sigma)));
+  f2_acc(h, l, f2sub(a.s1, f2splat(a.sigma)));
+  return f2_finish(h, f2add(l, f2add(a.e0, a.e1)));
+}
+// The pairs of kLanes neighbouring lanes added in a fixed butterfly (every lane of the warp
+// takes part); the sum in all of them.
+template <int kLanes>
+__device__ __forceinline__ float2 lanes_pair_sum(float2 P) {
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) {
+    const float a = __shfl_xor_sync(0xffffffffu, P.x, o), c = __shfl_xor_sync(0xffffffffu, P.y, o);
+    float t, u;
+    two_sum(P.x, a, t, u);
+    P.x = t;
+    P.y = P.y + c + u;
+  }
+  float h, l;
+  two_sum(P.x, P.y, h, l);
+  return make_float2(h, l);
+}
+
+// |x|^2 and, with kDot, <x, y> of two bf16 rows of d elements (16-byte aligned) as float
+// pairs, by the 16 lanes of a half-warp (hl = lane & 15): 16-byte chunks hl, hl + 16, ..,
+// two stages of two chunks in flight.  nx, ny: fp32 squared norms of the rows, good to
+// far better than 1 %, which give the sums' biases; a half whose sums leave the biases'
+// range (a norm that was not what it was taken for) starts over with TwoSum per product.  All
+// lanes of the warp call it together; `live` is false on a half without a row.  The two
+// halves' rows are independent.
+template <bool kDot>
+__device__ __forceinline__ void half_warp_row_sums(const uint4* x, const uint4* y, int d, float nx, float ny, int hl,
+                                                   bool live, float2& n2, float2& dot) {
+  const int nch = d / 8;
+  BiasedSum sn, sd;
+  bs_init(sn, pow2_ceil(4.04f * nx));
+  if (kDot) bs_init(sd, pow2_ceil(2.02f * (nx + ny)));
+  constexpr int kU = 2;  // chunks of a stage
+  auto load = [&](int k0, uint4 (&a)[kU], uint4 (&b)[kU]) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int k = k0 + 16 * u + hl;
+      const bool in = live && k < nch;
+      a[u] = in ? x[k] : make_uint4(0u, 0u, 0u, 0u);  // past the row's end: zeros, which add nothing
+      if (kDot) b[u] = in ? y[k] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  auto add = [&](const uint4 (&a)[kU], const uint4 (&b)[kU]) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w};
+#pragma unroll
+      for (int h = 0; h < 4; h += 2) {
+        const uint64_t x0 = bf16x2_f32x2(aw[h]), x1 = bf16x2_f32x2(aw[h + 1]);
+        biased_add(sn.s0, sn.e0, x0, x0);
+        biased_add(sn.s1, sn.e1, x1, x1);
+        if (kDot) {
+          const uint32_t bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
+          biased_add(sd.s0, sd.e0, x0, bf16x2_f32x2(bw[h]));
+          biased_add(sd.s1, sd.e1, x1, bf16x2_f32x2(bw[h + 1]));
+        }
+      }
+    }
+  };
+  uint4 xa[kU], ya[kU], xb[kU], yb[kU];
+  load(0, xa, ya);
+#pragma unroll 1
+  for (int k0 = 0; k0 < nch; k0 += 32 * kU) {
+    load(k0 + 16 * kU, xb, yb);
+    add(xa, ya);
+    load(k0 + 32 * kU, xa, ya);
+    add(xb, yb);
+  }
+  const uint16_t* xr = reinterpret_cast<const uint16_t*>(x);
+  const uint16_t* yr = reinterpret_cast<const uint16_t*>(y);
+  const bool tail = d % 8 != 0 && hl == 0 && live;  // the ragged end of the row, one lane per half
+  if (tail) {
+    for (int k = 8 * nch; k < d; ++k) {
+      const uint64_t xx = pack_f2((uint32_t)xr[k] << 16, 0u);
+      biased_add(sn.s0, sn.e0, xx, xx);
+      if (kDot) biased_add(sd.s0, sd.e0, xx, pack_f2((uint32_t)yr[k] << 16, 0u));
+    }
+  }
+  bool ok = !live || (bs_in_range(sn) && (!kDot || bs_in_range(sd)));
+  const uint32_t okm = __ballot_sync(0xffffffffu, ok);
+  const uint32_t half = (threadIdx.x & 16) ? 0xFFFF0000u : 0x0000FFFFu;
+  float2 pn = bs_pair(sn), pd = kDot ? bs_pair(sd) : make_float2(0.f, 0.f);
+  if ((okm & half) != half) {  // this half again, by TwoSum
+    uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
+#pragma unroll 1
+    for (int k = hl; k < nch; k += 16) {
+      const uint4 a = x[k];
+      uint4 b = make_uint4(0u, 0u, 0u, 0u);
+      if (kDot) b = y[k];
+      const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll 1
+      for (int h = 0; h < 4; ++h) {
+        const uint64_t xx = bf16x2_f32x2(aw[h]);
+        f2_acc(ns, ne, f2mul(xx, xx));
+        if (kDot) f2_acc(ds, de, f2mul(xx, bf16x2_f32x2(bw[h])));
+      }
+    }
+    if (tail) {
+      for (int k = 8 * nch; k < d; ++k) {
+        const uint64_t xx = pack_f2((uint32_t)xr[k] << 16, 0u);
+        f2_acc(ns, ne, f2mul(xx, xx));
+        if (kDot) f2_acc(ds, de, f2mul(xx, pack_f2((uint32_t)yr[k] << 16, 0u)));
+      }
+    }
+    pn = f2_finish(ns, ne);
+    pd = f2_finish(ds, de);
+  }
+  n2 = lanes_pair_sum<16>(pn);
+  dot = kDot ? lanes_pair_sum<16>(pd) : pd;
 }
 
 // One warp: |z|^2 of the row at element offset zrow of `base` and, if has_p, its dot with
@@ -668,9 +752,8 @@ struct LaunchCtx {
 };
 
 cudaError_t launch_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
-// with_norms: ws.nrm2 holds every row's fp32 squared norm (the similarity stage ran first)
-cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
-                               bool with_norms = false);
+// (ws.nrm2 holds every row's fp32 squared norm)
+cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
 cudaError_t launch_tree_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
 cudaError_t setup_tree_prep();
 cudaError_t launch_row_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
@@ -686,8 +769,6 @@ cudaError_t launch_tokens(const LaunchCtx& lc, const gpo_batch& b, const gpo_out
 // Records a message on the context (gpo_last_error).
 void note_error(gpo_ctx* ctx, const char* msg);
 
-// CTAs the fused kernel runs with for groups [g0, g1) (one group each when ng <= this).
-int fused_grid(const LaunchCtx& lc, const Sizes& sz);
 cudaError_t launch_fused(const LaunchCtx& lc, const CUtensorMap& map, const CUtensorMap& map32, const gpo_batch& b,
                          const gpo_outputs& o, const Sizes& sz, const Ws& ws, const Params& p);
 cudaError_t setup_fused();
