@@ -139,6 +139,7 @@ Ws workspace_views(void* base, const Layout& L) {
   w.edges = reinterpret_cast<int2*>(p + L.edges);
   w.e_adv = reinterpret_cast<float*>(p + L.e_adv);
   w.e_cor = reinterpret_cast<float*>(p + L.e_cor);
+  w.lab = nullptr;
   w.e_eff = reinterpret_cast<float*>(p + L.e_eff);
   w.e_mask = p + L.e_mask;
   w.tok_start = reinterpret_cast<int64_t*>(p + L.tok_start);
@@ -268,7 +269,7 @@ gpo_status gpo_create(gpo_ctx** out, const gpo_params* params) {
       return GPO_ERR_CUDA;
     }
   }
-  if (setup_sim_tc() != cudaSuccess || setup_groups() != cudaSuccess || setup_fused() != cudaSuccess ||
+  if (setup_sim_tc() != cudaSuccess || setup_sim_simt() != cudaSuccess || setup_groups() != cudaSuccess || setup_fused() != cudaSuccess ||
       setup_fused_f32() != cudaSuccess ||
       setup_tree_prep() != cudaSuccess || setup_loss() != cudaSuccess ||
       cudaMallocHost(&c->host_status, sizeof(uint32_t) * kStatusWords) != cudaSuccess) {
@@ -364,12 +365,13 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   pp.active = bud ? bud->active : nullptr;
   pp.budget = bud ? bud->budget : nullptr;
   pp.debug_timeout = (p.flags & GPO_FLAG_DEBUG_TIMEOUT) != 0;
-  const Ws ws = workspace_views(workspace, L);
+  Ws ws = workspace_views(workspace, L);
   LaunchCtx lc;
   lc.stream = static_cast<cudaStream_t>(stream);
   lc.num_sms = ctx->num_sms;
 
   const bool use_tc = b.emb_dtype == GPO_EMB_BF16 && !(p.flags & GPO_FLAG_SIMT_SIMILARITY) && sz.N > 0;
+  if (!use_tc) ws.lab = reinterpret_cast<int*>(ws.e_cor);
   const bool fused = use_tc && !(p.flags & GPO_FLAG_TILED) && sz.G > 0 && sz.maxn <= kFusedMaxStates;
   // fp32 embeddings, chain layout, small groups: the one-launch CUDA-core path
   const bool fused32 = b.emb_dtype == GPO_EMB_F32 && !b.parent && !bud && !(p.flags & GPO_FLAG_TILED) && sz.G > 0 &&
@@ -426,15 +428,18 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
     if (e == cudaSuccess && b.parent) e = stage("tree_prep", [&] { return launch_tree_prep(lc, b, sz, ws); });
     if (e == cudaSuccess) e = stage("prep", [&] { return launch_prep(lc, b, sz, ws); });
     if (e == cudaSuccess && sz.N > 0) {
-      // the fp32 norms of the threshold test come from the Gram tiles (tcgen05) or from
-      // row_stats (CUDA cores); eta takes compensated norms and parent dots (exact_stats),
-      // after the similarity stage so that the fp32 norms give the sums' biases
-      if (e == cudaSuccess && !use_tc) e = stage("row_stats", [&] { return launch_row_stats(lc, b, sz, ws); });
+      // the fp32 norms of the threshold test come from the Gram tiles (tcgen05), from the
+      // compensated statistics (fp32 embeddings, first then) or from row_stats; bf16 embeddings'
+      // statistics follow the similarity stage or row_stats, whose norms give their sums' biases
+      const bool exact_first = !use_tc && !bud && b.emb_dtype == GPO_EMB_F32;
+      auto exact = [&] { return launch_exact_stats(lc, b, sz, ws); };
+      if (exact_first) e = stage("exact_stats", exact);
+      else if (!use_tc) e = stage("row_stats", [&] { return launch_row_stats(lc, b, sz, ws); });
       if (e == cudaSuccess)
         e = stage("similarity", [&] {
           return use_tc ? launch_sim_tc(lc, map, b, sz, ws, pp) : launch_sim_simt(lc, b, sz, ws, pp);
         });
-      if (e == cudaSuccess && !bud) e = stage("exact_stats", [&] { return launch_exact_stats(lc, b, sz, ws); });
+      if (e == cudaSuccess && !bud && !exact_first) e = stage("exact_stats", exact);
       if (e == cudaSuccess) e = stage("groups", [&] { return launch_groups(lc, b, *out, sz, ws, pp); });
       if (e == cudaSuccess && !bud) e = stage("tokens", [&] { return launch_tokens(lc, b, *out, sz, ws); });
     }

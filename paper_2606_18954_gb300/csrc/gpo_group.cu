@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
   int16_t* ttown = tcown + al16(sizeof(int16_t) * (size_t)n) / sizeof(int16_t);
 
   for (int i = tid; i < n; i += nt) {
-    lab[i] = i;
+    lab[i] = ws.lab ? ws.lab[s0 + i] - s0 : i;
     const int2 m = ws.state_meta[s0 + i];
     dep[i] = (int16_t)m.y;
     if (tree) {
@@ -73,7 +73,9 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
   }
   __syncthreads();
 
-  // equivalence classes from the items' spanning forests, in the label forest lab
+  // equivalence classes: the CUDA-core similarity united the linked pairs in the batch's label
+  // forest (read above); the tensor-core one leaves the items' spanning forests, joined here
+  // in the label forest lab
   // (lab[x] <= x, within x's class): rounds of hooking over every listed pair (the larger of
   // the two current labels is pointed at the smaller, an atomic min) and shortcutting
   // (lab[x] = lab[lab[x]]) until no pair has unequal labels and every label is a root: then
@@ -81,7 +83,7 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
   // forest) finish the job if the rounds have not settled after kMaxRounds.
   // Items are dealt to warps (one item per warp at a time, lanes over its edges); the items'
   // edge counts are read once into shared memory (X, free until the group math).
-  const int nit = gi.nblk + gi.noff;  // the group's diagonal items, then its off-diagonal ones
+  const int nit = ws.lab ? 0 : gi.nblk + gi.noff;  // the group's diagonal items, then its off-diagonal ones
   auto item_at = [&](int k) { return k < gi.nblk ? gi.blk0 + k : gi.off0 + (k - gi.nblk); };
   int* ecnt = reinterpret_cast<int*>(X);
   const bool cached = !tree && (size_t)nit * sizeof(int) <= group_scratch_bytes(n);
@@ -89,7 +91,7 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
     for (int k = tid; k < nit; k += nt) ecnt[k] = min(ws.edge_count[item_at(k)], kEdgeCap);
   __syncthreads();
   const int lane = tid & 31, wid = tid >> 5, nwarp = nt >> 5;
-  bool settled = false;
+  bool settled = ws.lab != nullptr;
   for (int round = 0; round < kMaxRounds && !settled; ++round) {
     int ch = 0;
     for (int k = wid; k < nit; k += nwarp) {

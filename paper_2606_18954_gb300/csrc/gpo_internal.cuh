@@ -60,6 +60,8 @@ struct Ws {
   int2* edges;           // [max_items * kEdgeCap]
   float* e_adv;          // [N] A_dual per edge
   float* e_cor;          // [N] A_cor per edge
+  int* lab;              // [N] label forest of the CUDA-core similarity (in e_cor's place, which is
+                         // written once the labels are read; null on the tensor-core path)
   float* e_eff;          // [N] routed efficiency advantage per edge
   uint8_t* e_mask;       // [N]
   int64_t* tok_start;    // [N] first token of each edge
@@ -778,6 +780,7 @@ cudaError_t setup_fused_f32();
 cudaError_t launch_fused_f32(const LaunchCtx& lc, const gpo_batch& b, const gpo_outputs& o, const Sizes& sz,
                              const Ws& ws, const Params& p);
 cudaError_t setup_sim_tc();
+cudaError_t setup_sim_simt();
 cudaError_t setup_groups();
 size_t sim_tc_smem_bytes();
 size_t groups_smem_bytes(int maxn);

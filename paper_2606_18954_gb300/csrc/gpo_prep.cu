@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
       bad |= L < 1;
       sum += L;
       ws.state_meta[v] = make_int2(r, v - s + 1);
+      if (ws.lab) ws.lab[v] = v;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_prep_kernel(gpo_batch b, Si
       atomicMax(&end[x], i + 1);
     }
     ws.state_meta[s0 + i] = make_int2(g, d);
+    if (ws.lab) ws.lab[s0 + i] = s0 + i;
     ws.tree_par[s0 + i] = pp < 0 ? -1 : s0 + pp;
   }
   if (__syncthreads_or(bad)) {
@@ -356,8 +358,8 @@ cudaError_t launch_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz
 }
 
 // ---------------------------------------------------------------------------
-// K1a (CUDA-core similarity only): |z_v|^2 and 1/|z_v| with fp32 accumulation for the
-// threshold test, one warp per row (lane partial sums over a strided set of elements, then
+// K1a (CUDA-core similarity of bf16 embeddings, and of fp32 ones in gpo_layer_budget, which
+// needs no compensated statistics): |z_v|^2 and 1/|z_v| with fp32 accumulation for the threshold test, one warp per row (lane partial sums over a strided set of elements, then
 // a shuffle tree).  eta takes its norms from exact_stats instead.
 
 template <bool kBf16>
@@ -508,6 +510,10 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
       if (!isfinite(n2.x) || !isfinite(dot.x)) report(ws.status, GPO_ERR_NONFINITE, 3, v);
       ws.x_n2[v] = n2;
       ws.x_dot[v] = dot;
+      if (!kBf16) {  // the norms of the threshold test (bf16: from the similarity stage or row_stats)
+        ws.nrm2[v] = n2.x;
+        ws.rn[v] = n2.x > 0.f ? 1.0f / sqrtf(n2.x) : 0.f;
+      }
     }
   }
 }

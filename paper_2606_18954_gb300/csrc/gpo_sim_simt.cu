@@ -1,20 +1,52 @@
-// Cosine-similarity merge on the CUDA cores (fp32 embeddings; also selectable
-// for bf16 to cross-check the tensor-core kernel).  Same work items and same
-// per-item spanning-forest output as the tcgen05 kernel: GraphPO Sec. 4.2,
-// pairs of states of one group that are not ancestor-related and have
-// cosine >= kappa are linked.  fp32 fused multiply-add accumulation.
+// Cosine-similarity merge on the CUDA cores (fp32 embeddings; also selectable for bf16 to
+// cross-check the tensor-core kernel): GraphPO Sec. 4.2, pairs of states of one group that
+// are not ancestor-related and have cosine >= kappa are linked.  fp32 fused multiply-add
+// accumulation.
+//
+// One CTA per 64 x 32 tile of a work item (a 128-row block against up to 256 columns: two row
+// halves by eight column chunks; tiles left of a diagonal item's diagonal are empty).  Two
+// parts of 64 threads, each half of every stage's k: thread (ti, tj) = (t / 8, t % 8) of a part
+// owns the outputs of rows ti + 8 a and columns tj + 8 c (a < 8, c < NC), per four elements of
+// k one 16-byte chunk of each of its 8 rows and NC columns and 32 NC fma; the second part's
+// sums are added to the first's through shared memory.  Rows are staged as they lie in memory,
+// kKc elements at a time (row stride kKc + 4 floats: eight consecutive rows fall in eight
+// different 16-byte bank groups), in two buffers filled by cp.async while the other one is
+// multiplied.  NC = 2 or 4 column chunks of 8 by the tile's valid columns, so that a group of a
+// few states more than a multiple of 32 does not pay whole tiles for them.  The linked pairs of
+// a tile are united in shared memory, then one union per non-root state in the batch's label
+// forest (ws.lab).
+//
+// Bound by fp32 issue (64 % of the slots while an SM has work, three quarters of them fma):
+// 64 groups of 257 states, d = 1024 take 184 us, of which the fma of their upper-triangle
+// tiles are 78 us of the fp32 pipe.  Before, one CTA of 256 threads per item with scalar loads
+// transposed into shared memory: 795 us.  The same tile with 64 threads and whole k, one wave
+// of long CTAs: 238 us; with four parts 205 us; packed f32x2 fma 256 us.
 #include "gpo_internal.cuh"
 
 namespace gpo {
 
 namespace {
 
-constexpr int kThreads = 256;          // 16 x 16 threads, each 8 rows x 16 columns
-constexpr int kKc = 16;                // k-chunk staged in shared memory
-constexpr int kSlots = kTileM + kTileN;
+constexpr int kTile = 64, kCols = 32;  // rows and columns of a CTA's tile
+constexpr int kPart = 64;              // threads of one part
+constexpr int kParts = 2;              // parts: each half of every stage's k
+constexpr int kThreads = kParts * kPart;
+constexpr int kKc = 32;                // k elements of a stage
+constexpr int kLd = kKc + 4;           // row stride in shared memory (floats)
+constexpr int kSubs = 16;              // tiles of a work item: 2 row halves x 8 column chunks
+static_assert(kTileM == 2 * kTile && kTileN == 8 * kCols && kTile == 2 * kCols, "tiles of a work item");
 
-__device__ __forceinline__ int sfind(int* p, int x) {
-  volatile int* vp = p;
+struct SimtSmem {
+  alignas(16) float A[2][kTile * kLd];
+  alignas(16) float B[2][kCols * kLd];
+  float rrn[kTile], crn[kCols];        // 1 / |z| of the rows and columns
+  int rend[kTile];                     // first comparable column right of the row (state index)
+  int rdep[kTile], cdep[kCols];        // depths
+  int lp[kTile + kCols];               // label forest of the tile's rows, then columns
+};
+
+__device__ __forceinline__ int find_root(const int* p, int x) {
+  const volatile int* vp = p;
   while (true) {
     const int y = vp[x];
     if (y == x) return x;
@@ -22,10 +54,11 @@ __device__ __forceinline__ int sfind(int* p, int x) {
   }
 }
 
-__device__ __forceinline__ void sunion(int* p, int a, int b) {
+// Hook the larger root under the smaller one; parent[x] <= x always holds.
+__device__ __forceinline__ void unite(int* p, int a, int b) {
   while (true) {
-    a = sfind(p, a);
-    b = sfind(p, b);
+    a = find_root(p, a);
+    b = find_root(p, b);
     if (a == b) return;
     if (a > b) {
       const int t = a;
@@ -36,214 +69,195 @@ __device__ __forceinline__ void sunion(int* p, int a, int b) {
   }
 }
 
-template <bool kBf16>
-__device__ __forceinline__ float ld_elem(const void* base, int64_t i) {
-  if (kBf16) return __uint_as_float((uint32_t)(reinterpret_cast<const uint16_t*>(base)[i]) << 16);
-  return reinterpret_cast<const float*>(base)[i];
+// 16 bytes from global to shared memory, of which `bytes` are read and the rest zeros.
+__device__ __forceinline__ void cp_async16(float* dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kLeft>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(kLeft) : "memory");
 }
 
-constexpr int kSmall = 64;   // rows and columns of a small item
-constexpr int kKs = 32;      // k-chunk of a small item (kKs x kSmall floats fit in As and in Bs)
-static_assert(kKs * kSmall <= kKc * (kTileM + 4) && kKs * kSmall <= kKc * (kTileN + 4), "small-item staging");
-
-// A small item: the same products, pair test and unions as the general path below, with
-// every thread on a 4 x 4 micro-tile of the 64 x 64 block (all 256 threads busy) and
-// k-chunks of kKs elements (fewer barriers and load round trips per item).  As / Bs are
-// the general path's staging arrays, viewed as [kKs][kSmall].
+// Elements [k0, k0 + kKc) of rows [row0, row0 + nrows) into dst (zeros past d; rows past
+// nrows are not written, their outputs are not read).
 template <bool kBf16>
-__device__ __forceinline__ void small_item(const gpo_batch& b, const Sizes& sz, const Item& item, int nrows, int send,
-                                           float* As, float* Bs, const int* rm_roll, const int* rm_depth,
-                                           const int* rm_end, const float* rm_rn, const int* cm_roll,
-                                           const int* cm_depth, const float* cm_rn, int* lp, bool tree, float kappa,
-                                           int rule) {
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // columns 4 tx.., rows 4 ty..
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int k0 = 0; k0 < sz.d; k0 += kKs) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < kKs * nrows; e += kThreads) {
-      const int r = e / kKs, k = e % kKs;
-      const int row = item.row0 + r;
-      As[k * kSmall + r] = (row < send && k0 + k < sz.d) ? ld_elem<kBf16>(b.emb, (int64_t)row * sz.stride + k0 + k) : 0.f;
-    }
-    for (int e = threadIdx.x; e < kKs * item.ncols; e += kThreads) {
-      const int c = e / kKs, k = e % kKs;
-      Bs[k * kSmall + c] = k0 + k < sz.d ? ld_elem<kBf16>(b.emb, (int64_t)(item.col0 + c) * sz.stride + k0 + k) : 0.f;
-    }
-    __syncthreads();
-    if (ty * 4 < nrows && tx * 4 < item.ncols) {
-      const int kn = min(kKs, sz.d - k0);
-      for (int k = 0; k < kn; ++k) {
-        const float4 a = *reinterpret_cast<const float4*>(As + k * kSmall + ty * 4);
-        const float4 bv = *reinterpret_cast<const float4*>(Bs + k * kSmall + tx * 4);
-        const float av[4] = {a.x, a.y, a.z, a.w}, bw[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bw[j], acc[i][j]);
+__device__ __forceinline__ void stage_rows(float* dst, const void* emb, int64_t stride, int d, int row0, int nrows,
+                                           int k0) {
+  constexpr int kCh = kKc / 4;  // 16-byte chunks of a staged row
+  for (int e = threadIdx.x; e < nrows * kCh; e += kThreads) {
+    const int r = e / kCh, k = k0 + 4 * (e % kCh);
+    const int valid = max(0, min(4, d - k));
+    float* to = dst + r * kLd + 4 * (e % kCh);
+    const int64_t at = (int64_t)(row0 + r) * stride + (valid > 0 ? k : 0);
+    if (kBf16) {
+      const uint16_t* from = reinterpret_cast<const uint16_t*>(emb) + at;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (valid == 4) {  // 8-byte aligned: rows on 16 bytes, k a multiple of 4
+        const uint2 w = *reinterpret_cast<const uint2*>(from);
+        v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16),
+                        __uint_as_float(w.y & 0xFFFF0000u));
+      } else if (valid > 0) {
+        v.x = __uint_as_float((uint32_t)from[0] << 16);
+        if (valid > 1) v.y = __uint_as_float((uint32_t)from[1] << 16);
+        if (valid > 2) v.z = __uint_as_float((uint32_t)from[2] << 16);
       }
+      *reinterpret_cast<float4*>(to) = v;
+    } else {
+      cp_async16(to, reinterpret_cast<const float*>(emb) + at, 4 * valid);
     }
   }
+}
+
+// The tile's products (8 NC columns), pair test and links in sm.lp.
+template <bool kBf16, int NC>
+__device__ __forceinline__ void tile_links(SimtSmem& sm, const gpo_batch& b, const Sizes& sz, int row0, int nr,
+                                           int col0, int nc, float kappa, int rule) {
+  const int t = threadIdx.x % kPart, part = threadIdx.x / kPart, ti = t >> 3, tj = t & 7;
+  const int cr = col0 - row0;                    // columns that are rows of the tile too
+  const bool shared = cr + nc <= nr;             // are read from A
+  float acc[8][NC];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[a][c] = 0.f;
+  auto stage = [&](int k0, int buf) {
+    stage_rows<kBf16>(sm.A[buf], b.emb, sz.stride, sz.d, row0, nr, k0);
+    if (!shared) stage_rows<kBf16>(sm.B[buf], b.emb, sz.stride, sz.d, col0, nc, k0);
+    cp_async_commit();
+  };
+  const int nk = (sz.d + kKc - 1) / kKc;
+  stage(0, 0);
+#pragma unroll 1
+  for (int s = 0; s < nk; ++s) {
+    const int buf = s & 1;
+    if (s + 1 < nk) stage((s + 1) * kKc, buf ^ 1);
+    else cp_async_commit();  // (an empty group, so that the wait below always leaves one)
+    cp_async_wait<1>();
+    __syncthreads();
+    const int kp = part * (kKc / kParts);
+    const float* A = sm.A[buf] + ti * kLd + kp;
+    const float* B = (shared ? sm.A[buf] + cr * kLd : sm.B[buf]) + tj * kLd + kp;
+#pragma unroll 1
+    for (int k = 0; k < kKc / kParts; k += 4) {
+      float4 x[8], y[NC];
+#pragma unroll
+      for (int a = 0; a < 8; ++a) x[a] = *reinterpret_cast<const float4*>(A + 8 * a * kLd + k);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) y[c] = *reinterpret_cast<const float4*>(B + 8 * c * kLd + k);
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          float s4 = acc[a][c];
+          s4 = fmaf(x[a].x, y[c].x, s4);
+          s4 = fmaf(x[a].y, y[c].y, s4);
+          s4 = fmaf(x[a].z, y[c].z, s4);
+          s4 = fmaf(x[a].w, y[c].w, s4);
+          acc[a][c] = s4;
+        }
+    }
+    __syncthreads();  // the buffer is refilled two stages on
+  }
+  // the other parts' sums, added to the first's in part order
+  float* ps = &sm.A[0][0];
+  static_assert(sizeof(sm.A) >= sizeof(float) * 8 * 4 * kPart * (kParts - 1), "partial sums");
+  if (part > 0) {
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) ps[(((part - 1) * 8 + a) * NC + c) * kPart + t] = acc[a][c];
+  }
   __syncthreads();
+  if (part > 0) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = ty * 4 + i;
-    if (r >= nrows || rm_roll[r] < 0) continue;
-    const int row = item.row0 + r;
+  for (int q = 0; q < kParts - 1; ++q)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = tx * 4 + j;
-      const int col = item.col0 + c;
-      // comparable: not the row's own rollout (tree layout: outside the row's subtree)
-      if (c >= item.ncols || col <= row || (tree ? col < rm_end[r] : cm_roll[c] == rm_roll[r])) continue;
-      if (rule == GPO_MERGE_SAME_DEPTH && cm_depth[c] != rm_depth[r]) continue;
-      if (acc[i][j] * rm_rn[r] * cm_rn[c] >= kappa) {
-        const int sc = (col < item.row0 + kTileM) ? col - item.row0 : kTileM + (col - item.col0);
-        sunion(lp, r, sc);
-      }
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[a][c] += ps[((q * 8 + a) * NC + c) * kPart + t];
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    const int r = ti + 8 * a;
+    if (r >= nr) continue;
+    const float rn = sm.rrn[r];
+    const int re = sm.rend[r], di = sm.rdep[r];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int q = tj + 8 * c;
+      // comparable: right of the row and past its own rollout (tree layout: its subtree)
+      if (q >= nc || col0 + q < re) continue;
+      if (rule == GPO_MERGE_SAME_DEPTH && sm.cdep[q] != di) continue;
+      if (acc[a][c] * rn * sm.crn[q] >= kappa) unite(sm.lp, r, cr + q < kTile ? cr + q : kTile + q);
     }
   }
 }
 
 template <bool kBf16>
 __global__ void __launch_bounds__(kThreads) sim_simt_kernel(gpo_batch b, Sizes sz, Ws ws, float kappa, int rule) {
-  __shared__ __align__(16) float As[kKc][kTileM + 4];
-  __shared__ __align__(16) float Bs[kKc][kTileN + 4];
-  __shared__ int lp[kSlots];
-  __shared__ int cm_roll[kTileN], cm_depth[kTileN];
-  __shared__ float cm_rn[kTileN];
-  __shared__ int rm_roll[kTileM], rm_depth[kTileM], rm_end[kTileM];
-  __shared__ float rm_rn[kTileM];
-  __shared__ int edge_n;
+  extern __shared__ __align__(16) unsigned char simt_smem[];
+  SimtSmem& sm = *reinterpret_cast<SimtSmem*>(simt_smem);
   uint32_t* st = ws.status;
-  const bool tree = ws.tree_end != nullptr;
+  const int it = blockIdx.x / kSubs, sub = blockIdx.x % kSubs;
   const int nitems = (int)*((volatile uint32_t*)&st[kStItems]);
-  if (aborted(st)) return;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  for (int i = threadIdx.x; i < kSlots; i += kThreads) lp[i] = i;
-
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const Item item = ws.items[it];
-    const GroupInfo gi = ws.groups[item.group];
-    const int send = gi.s0 + gi.n;
-    __syncthreads();
-    for (int c = threadIdx.x; c < kTileN; c += kThreads) {
-      if (c < item.ncols) {
-        const int2 mt = ws.state_meta[item.col0 + c];
-        cm_roll[c] = mt.x;
-        cm_depth[c] = mt.y;
-        cm_rn[c] = ws.rn[item.col0 + c];
+  if (it >= nitems || aborted(st)) return;
+  const Item item = ws.items[it];
+  const GroupInfo gi = ws.groups[item.group];
+  const int send = gi.s0 + gi.n;
+  const int row0 = item.row0 + kTile * (sub & 1), col0 = item.col0 + kCols * (sub >> 1);
+  const int nr = min(kTile, send - row0), nc = min(kCols, item.col0 + item.ncols - col0);
+  if (nr <= 0 || nc <= 0 || col0 < row0) return;
+  const bool tree = ws.tree_end != nullptr;
+  {
+    const int x = threadIdx.x;
+    static_assert(kThreads >= kTile, "one row per thread");
+    if (x < kTile) sm.lp[x] = x;
+    if (x < nr) {
+      const int2 mt = ws.state_meta[row0 + x];
+      sm.rrn[x] = ws.rn[row0 + x];
+      sm.rdep[x] = mt.y;
+      sm.rend[x] = tree ? ws.tree_end[row0 + x] : b.rollout_step_off[mt.x + 1];
+    }
+    if (x < kCols) {
+      sm.lp[kTile + x] = kTile + x;
+      if (x < nc) {
+        sm.crn[x] = ws.rn[col0 + x];
+        sm.cdep[x] = ws.state_meta[col0 + x].y;
       }
     }
-    for (int r = threadIdx.x; r < kTileM; r += kThreads) {
-      const int row = item.row0 + r;
-      if (row < send) {
-        const int2 mt = ws.state_meta[row];
-        rm_roll[r] = mt.x;
-        rm_depth[r] = mt.y;
-        rm_rn[r] = ws.rn[row];
-        rm_end[r] = tree ? ws.tree_end[row] : 0;
-      } else {
-        rm_roll[r] = -1;
-      }
-    }
-    if (threadIdx.x == 0) edge_n = 0;
-
-    const int nrows = min(kTileM, send - item.row0);
-    if (nrows <= kSmall && item.ncols <= kSmall) {
-      // a small item (groups of at most 64 states): every thread one 4 x 4 micro-tile of the
-      // 64 x 64 block, k-chunks of kKs staged at once
-      small_item<kBf16>(b, sz, item, nrows, send, &As[0][0], &Bs[0][0], rm_roll, rm_depth, rm_end, rm_rn, cm_roll,
-                        cm_depth, cm_rn, lp, tree, kappa, rule);
-    } else {
-    float acc[8][16];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < 16; ++j) acc[i][j] = 0.f;
-    // only the tile's valid rows and columns are staged and multiplied (a thread's rows
-    // and columns past them accumulate stale values that the epilogue never reads)
-    const bool busy = ty * 8 < nrows && tx * 16 < item.ncols;
-
-    for (int k0 = 0; k0 < sz.d; k0 += kKc) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < kKc * nrows; e += kThreads) {
-        const int r = e / kKc, k = e % kKc;
-        const int row = item.row0 + r;
-        As[k][r] = (row < send && k0 + k < sz.d) ? ld_elem<kBf16>(b.emb, (int64_t)row * sz.stride + k0 + k) : 0.f;
-      }
-      for (int e = threadIdx.x; e < kKc * item.ncols; e += kThreads) {
-        const int c = e / kKc, k = e % kKc;
-        Bs[k][c] = (c < item.ncols && k0 + k < sz.d)
-                       ? ld_elem<kBf16>(b.emb, (int64_t)(item.col0 + c) * sz.stride + k0 + k)
-                       : 0.f;
-      }
-      __syncthreads();
-      if (busy) {
-#pragma unroll 4
-      for (int k = 0; k < kKc; ++k) {
-        float a[8], bv[16];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) a[i] = As[k][ty * 8 + i];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) bv[j] = Bs[k][tx * 16 + j];
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-          for (int j = 0; j < 16; ++j) acc[i][j] = fmaf(a[i], bv[j], acc[i][j]);
-      }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = ty * 8 + i;
-      const int row = item.row0 + r;
-      if (rm_roll[r] < 0) continue;
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int c = tx * 16 + j;
-        const int col = item.col0 + c;
-        // comparable: not the row's own rollout (tree layout: outside the row's subtree)
-        if (c >= item.ncols || col <= row || (tree ? col < rm_end[r] : cm_roll[c] == rm_roll[r])) continue;
-        if (rule == GPO_MERGE_SAME_DEPTH && cm_depth[c] != rm_depth[r]) continue;
-        if (acc[i][j] * rm_rn[r] * cm_rn[c] >= kappa) {
-          const int sc = (col < item.row0 + kTileM) ? col - item.row0 : kTileM + (col - item.col0);
-          sunion(lp, r, sc);
-        }
-      }
-    }
-    }
-    __syncthreads();
-    int2* out = ws.edges + (size_t)it * kEdgeCap;
-    for (int s = threadIdx.x; s < kSlots; s += kThreads) {
-      const int root = sfind(lp, s);
-      if (root != s) {
-        const int gs = s < kTileM ? item.row0 + s : item.col0 + (s - kTileM);
-        const int gr = root < kTileM ? item.row0 + root : item.col0 + (root - kTileM);
-        const int k = atomicAdd(&edge_n, 1);
-        if (k < kEdgeCap) out[k] = make_int2(gr, gs);
-      }
-    }
-    __syncthreads();
-    for (int s = threadIdx.x; s < kSlots; s += kThreads) lp[s] = s;
-    if (threadIdx.x == 0) ws.edge_count[it] = min(edge_n, kEdgeCap);
+  }
+  if (nc > 16) tile_links<kBf16, 4>(sm, b, sz, row0, nr, col0, nc, kappa, rule);
+  else tile_links<kBf16, 2>(sm, b, sz, row0, nr, col0, nc, kappa, rule);
+  __syncthreads();
+  // (a column that is a row of the tile has the row's slot)
+  for (int x = threadIdx.x; x < kTile + kCols; x += kThreads) {
+    const int root = find_root(sm.lp, x);
+    if (root == x) continue;
+    const int v = x < kTile ? row0 + x : col0 + (x - kTile);
+    const int u = root < kTile ? row0 + root : col0 + (root - kTile);
+    if (GPO_BOUNDS(st, v, sz.N, kWhereEdges) && GPO_BOUNDS(st, u, sz.N, kWhereEdges)) unite(ws.lab, u, v);
   }
 }
 
 }  // namespace
 
+cudaError_t setup_sim_simt() {
+  cudaError_t e = cudaFuncSetAttribute(sim_simt_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(SimtSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(sim_simt_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(SimtSmem));
+  return e;
+}
+
 cudaError_t launch_sim_simt(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                             const Params& p) {
-  int grid = ws.max_items < 4 * lc.num_sms ? ws.max_items : 4 * lc.num_sms;
-  if (grid < 1) return cudaSuccess;
+  if (ws.max_items < 1) return cudaSuccess;
+  const unsigned grid = (unsigned)ws.max_items * kSubs;  // max_items < 2^27 (layout)
   if (b.emb_dtype == GPO_EMB_BF16)
-    sim_simt_kernel<true><<<grid, kThreads, 0, lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule);
+    sim_simt_kernel<true><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule);
   else
-    sim_simt_kernel<false><<<grid, kThreads, 0, lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule);
+    sim_simt_kernel<false><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule);
   return cudaGetLastError();
 }
 
