@@ -787,7 +787,7 @@ size_t groups_smem_bytes(int maxn);
 
 // ------------------------------------------------------------------ policy loss
 
-constexpr int kLossTile = 4096;        // tokens per tile of the loss kernel
+constexpr int kLossTile = 512;         // tokens per tile of the loss kernel (one warp's step)
 constexpr int kLossMaxBlocks = 1024;   // CTAs of one loss launch at most (reduction scratch)
 constexpr int kLossPlanHead = 256;     // bytes: status words, then the group count and the ticket
 constexpr int kLossWordGroups = kStatusWords, kLossWordTicket = kStatusWords + 1;

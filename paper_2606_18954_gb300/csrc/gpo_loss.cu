@@ -6,16 +6,19 @@
 //             rollout, or per group in the tree layout) and counts the groups with
 //             states; loss_weights_kernel: every edge's token weight 1/(G' |E_g| |e|)
 //             and the edge holding the first token of every tile of kLossTile tokens.
-//   loss      token_loss_kernel: persistent CTAs over token tiles; a tile's edges (first
-//             token, weight x advantages; at most one per token) are staged in shared
-//             memory with a token -> edge map of the tile; each thread takes four 16-byte
-//             chunks of tokens (coalesced across the CTA; all four loaded before the
-//             edges are staged) and reads each token's edge from the map; per token the
-//             ratio, the
-//             clipped surrogate, the k3 KL estimate, the gradient (one 16-byte store per
-//             chunk); sums in fp32 per tile, fp64 across tiles, per-CTA partials combined
-//             by the last CTA in a fixed order (deterministic).
-// HBM-bound: 12 bytes per token (16 with the KL term) plus ~16 bytes per edge.
+//   loss      token_loss_kernel: every warp walks tiles of kLossTile tokens by itself, with no
+//             barrier of its CTA: its lanes' tokens first (four 16-byte chunks per array,
+//             all in flight), then the tile's edges (at most one per token) into the warp's part
+//             of shared memory, the edge of every chunk's first token from a count of the
+//             edges that start up to it (one shared-memory atomic per edge, one warp scan);
+//             per token the ratio, the clipped surrogate, the k3 KL estimate, the gradient
+//             (one 16-byte store per chunk); sums in fp32 per tile, float pairs across tiles,
+//             per-CTA partials combined by the last CTA in a fixed order (deterministic).
+// 12 bytes per token (16 with the KL term) plus ~16 bytes per edge; bound by issue (57 % of the
+// slots) and by the latency of a tile's loads.  While a warp waits for its tokens or edges
+// the SM's others compute, which CTA-wide steps of 4096 tokens with three barriers each did
+// not allow: 38.3 M tokens in the split form with the KL term 183 -> 128 us (4.8 TB/s), 4.7 M
+// in the dual form 27.3 -> 23.2 us.  Tiles of 256 tokens: 132 / 25.2 us.
 #include "gpo_internal.cuh"
 
 namespace gpo {
@@ -24,8 +27,9 @@ namespace {
 
 constexpr int kPlanThreads = 256;
 constexpr int kLossThreads = 256;
-constexpr int kLossChunks = kLossTile / (4 * kLossThreads);  // 16-byte chunks per thread and tile
-static_assert(kLossChunks * 4 * kLossThreads == kLossTile, "loss tile shape");
+constexpr int kLossWarps = kLossThreads / 32;
+constexpr int kLossChunks = kLossTile / (4 * 32);  // 16-byte chunks per lane and tile
+static_assert(kLossChunks * 4 * 32 == kLossTile, "loss tile shape");
 
 __device__ __forceinline__ int64_t warp_incl_scan(int64_t x, int lane) {
 #pragma unroll
@@ -141,26 +145,34 @@ __global__ void __launch_bounds__(256) loss_weights_kernel(Sizes sz, LossPlan lp
   }
 }
 
-// e^x - 1 (em1) and e^x - 1 - x (k3) of x = log pi_ref - log pi_theta: for |x| < 1/2 from
+// e^x - 1 (em1) and e^x - 1 - x (k3) of four x = log pi_ref - log pi_theta: for |x| < 1/2 from
 // the Taylor series of e^x (terms up to x^10 / 10!: truncation below 1e-10 relative), else
 // from the fast exponential (|e^x - 1| >= 0.39 and k3 >= 0.1 there, so its few-ulp error
-// stays a few ulp)
-__device__ __forceinline__ void kl_terms(float x, float& em1, float& k3) {
-  if (fabsf(x) < 0.5f) {
+// stays a few ulp), behind one branch for the four
+__device__ __forceinline__ void kl_terms(const float (&x)[4], float (&em1)[4], float (&k3)[4]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const float v = x[c];
     float p = 1.f / 3628800.f;
-    p = fmaf(p, x, 1.f / 362880.f);
-    p = fmaf(p, x, 1.f / 40320.f);
-    p = fmaf(p, x, 1.f / 5040.f);
-    p = fmaf(p, x, 1.f / 720.f);
-    p = fmaf(p, x, 1.f / 120.f);
-    p = fmaf(p, x, 1.f / 24.f);
-    p = fmaf(p, x, 1.f / 6.f);
-    p = fmaf(p, x, 0.5f);
-    k3 = x * x * p;
-    em1 = x + k3;
-  } else {
-    em1 = __expf(x) - 1.f;
-    k3 = em1 - x;
+    p = fmaf(p, v, 1.f / 362880.f);
+    p = fmaf(p, v, 1.f / 40320.f);
+    p = fmaf(p, v, 1.f / 5040.f);
+    p = fmaf(p, v, 1.f / 720.f);
+    p = fmaf(p, v, 1.f / 120.f);
+    p = fmaf(p, v, 1.f / 24.f);
+    p = fmaf(p, v, 1.f / 6.f);
+    p = fmaf(p, v, 0.5f);
+    k3[c] = v * v * p;
+    em1[c] = v + k3[c];
+  }
+  if (!(fmaxf(fmaxf(fabsf(x[0]), fabsf(x[1])), fmaxf(fabsf(x[2]), fabsf(x[3]))) < 0.5f)) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (!(fabsf(x[c]) < 0.5f)) {
+        em1[c] = __expf(x[c]) - 1.f;
+        k3[c] = em1[c] - x[c];
+      }
+    }
   }
 }
 
@@ -175,18 +187,166 @@ __device__ __forceinline__ bool surrogate(float r, float rc, float wa, float& f,
   return !take;
 }
 
-// Shared memory of one CTA: the tile's edges (at most one per token)
+// A warp's part of shared memory: its tile's edges (at most one per token)
+template <bool kSplit, bool kKL>
+struct LossWarp {
+  alignas(16) int count[kLossTile / 4];   // edges starting up to each chunk's first token
+  int16_t start[kLossTile + 4];           // first token of each edge, relative to the tile
+  float wa[kLossTile + 1];                // w A (dual) or w A_cor (split)
+  float we[kSplit ? kLossTile + 1 : 1];   // split: w lambda m_eff A_eff
+  float w[kKL ? kLossTile + 1 : 1];       // KL: w
+};
+
 template <bool kSplit, bool kKL>
 struct LossSmem {
-  uint16_t map[kLossTile];                // edge (tile-local) of every token of the tile
-  int16_t start[kLossTile + 2];           // first token of each edge, relative to the tile
-  float wa[kLossTile];                    // w A (dual) or w A_cor (split)
-  float we[kSplit ? kLossTile : 1];       // split: w lambda m_eff A_eff
-  float w[kKL ? kLossTile : 1];           // KL: w
-  float2 red[kLossThreads / 32][3];
-  long long redn[kLossThreads / 32];
+  LossWarp<kSplit, kKL> warp[kLossWarps];
+  float2 red[kLossWarps][3];
+  long long redn[kLossWarps];
   int last;
 };
+
+// One tile of one warp: the sums of its tokens' policy terms (pg), KL terms (kl) and ratios (rs)
+// and the count of clipped ones, per lane; their gradients.  kFull: all kLossTile tokens exist
+// (tn of them otherwise), which leaves out a comparison and a select per token and sum.
+template <bool kSplit, bool kKL, bool kFull>
+__device__ __forceinline__ void tile_loss(const LossArgs& a, const LossPlan& lp, LossWarp<kSplit, kKL>& ws,
+                                          int64_t tile, int tn, int lane, float& pg, float& kl, float& rs,
+                                          int& nclip) {
+  const int64_t t0 = tile * kLossTile;
+  // the lane's token chunks first (streaming loads, all in flight together), then the tile's
+  // edges: the memory latencies overlap
+  float x[kLossChunks][4], y[kLossChunks][4], z[kLossChunks][4];
+#pragma unroll
+  for (int k = 0; k < kLossChunks; ++k) {
+    const int rel = 4 * (lane + 32 * k);
+    const int64_t q = t0 + rel;
+    if (kFull || rel + 4 <= tn) {
+      const float4 u = __ldcs(reinterpret_cast<const float4*>(a.logp + q));
+      const float4 v = __ldcs(reinterpret_cast<const float4*>(a.old_logp + q));
+      x[k][0] = u.x, x[k][1] = u.y, x[k][2] = u.z, x[k][3] = u.w;
+      y[k][0] = v.x, y[k][1] = v.y, y[k][2] = v.z, y[k][3] = v.w;
+      if (kKL) {
+        const float4 w4 = __ldcs(reinterpret_cast<const float4*>(a.ref_logp + q));
+        z[k][0] = w4.x, z[k][1] = w4.y, z[k][2] = w4.z, z[k][3] = w4.w;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const bool in = rel + c < tn;
+        x[k][c] = in ? a.logp[q + c] : 0.f;
+        y[k][c] = in ? a.old_logp[q + c] : 0.f;
+        if (kKL) z[k][c] = in ? a.ref_logp[q + c] : 0.f;
+      }
+    }
+  }
+  // edges [e_lo, e_hi] hold the tile's tokens (each edge has >= 1 token: at most kLossTile)
+  const int e_lo = min(max(lp.tile_edge[tile], 0), a.N - 1);
+  const int e_hi = min(max(lp.tile_edge[tile + 1], e_lo), min(a.N - 1, e_lo + kLossTile - 1));
+  const int ne = e_hi - e_lo + 1;
+  __syncwarp();  // the previous tile's readers are done
+#pragma unroll
+  for (int i = 0; i < kLossChunks; ++i) ws.count[lane + 32 * i] = 0;
+  __syncwarp();
+  for (int j = lane; j <= ne; j += 32) {
+    const int64_t st = lp.start[e_lo + j] - t0;
+    const int rel = (int)max(min(st, (int64_t)kLossTile), (int64_t)0);  // clamped to the tile
+    ws.start[j] = (int16_t)rel;
+    if (j < ne) {
+      const float w = a.norm_token ? a.inv_t : lp.w[e_lo + j];
+      ws.wa[j] = w * a.adv[e_lo + j];
+      if (kSplit) ws.we[j] = a.mask[e_lo + j] ? w * (a.lambda * a.eff[e_lo + j]) : 0.f;
+      if (kKL) ws.w[j] = w;
+      const int chunk = (rel + 3) >> 2;  // the first chunk whose first token it holds
+      if (j > 0 && chunk < kLossTile / 4) atomicAdd(&ws.count[chunk], 1);
+    } else {
+      ws.start[j + 1] = (int16_t)kLossTile;  // (past the end, read with the last edge)
+    }
+  }
+  __syncwarp();
+  {  // inclusive scan of the chunks' counts: the edge (tile-local) of each chunk's first token
+    int c[kLossChunks], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kLossChunks; ++i) {
+      sum += ws.count[kLossChunks * lane + i];
+      c[i] = sum;
+    }
+    const int own = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, sum, o);
+      if (lane >= o) sum += u;
+    }
+#pragma unroll
+    for (int i = 0; i < kLossChunks; ++i) ws.count[kLossChunks * lane + i] = c[i] + sum - own;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < kLossChunks; ++k) {
+    const int rel = 4 * (lane + 32 * k);  // first token of this chunk in the tile
+    if (!kFull && rel >= tn) continue;
+    // the chunk's edges: j0 holds its first token, j0 + 1 the tokens from s1 on; a third one
+    // only where j0 + 1 is shorter than 3 tokens
+    const int j0 = min(ws.count[lane + 32 * k], ne - 1), j1 = min(j0 + 1, ne - 1);
+    const int s1 = ws.start[j0 + 1] - rel;
+    const bool third = ws.start[j0 + 2] - rel < 4;
+    const float wa0 = ws.wa[j0], wa1 = ws.wa[j1];
+    const float we0 = kSplit ? ws.we[j0] : 0.f, we1 = kSplit ? ws.we[j1] : 0.f;
+    const float w0 = kKL ? ws.w[j0] : 0.f, w1 = kKL ? ws.w[j1] : 0.f;
+    float wa[4], we[4], w[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      wa[c] = c < s1 ? wa0 : wa1;
+      we[c] = c < s1 ? we0 : we1;
+      w[c] = c < s1 ? w0 : w1;
+    }
+    if (third) {
+      int j = j0;
+#pragma unroll
+      for (int c = 1; c < 4; ++c) {  // (every edge has a token: at most one starts per token)
+        if (j + 1 < ne && ws.start[j + 1] <= rel + c) ++j;
+        wa[c] = ws.wa[j];
+        if (kSplit) we[c] = ws.we[j];
+        if (kKL) w[c] = ws.w[j];
+      }
+    }
+    float gr[4], em1[4], k3[4];
+    if (kKL) {
+      const float d[4] = {z[k][0] - x[k][0], z[k][1] - x[k][1], z[k][2] - x[k][2], z[k][3] - x[k][3]};
+      kl_terms(d, em1, k3);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const bool in = kFull || rel + c < tn;  // (tokens past the tile's end take some edge's weight)
+      const float r = __expf(x[k][c] - y[k][c]);
+      const float rc = fminf(fmaxf(r, a.lo), a.hi);
+      float f, df;
+      const bool clipped = surrogate(r, rc, wa[c], f, df);
+      if (kSplit) {
+        float f2, df2;
+        surrogate(r, rc, we[c], f2, df2);
+        f += f2;
+        df += df2;
+      }
+      float g = -df;
+      if (kKL) {
+        kl = in ? fmaf(w[c], k3[c], kl) : kl;
+        g = fmaf(-a.beta * w[c], em1[c], g);  // beta w (1 - e^x)
+      }
+      if (in) {
+        pg += f;
+        rs += r;
+        nclip += clipped ? 1 : 0;
+      }
+      gr[c] = g;
+    }
+    if (a.grad) {
+      const int64_t q = t0 + rel;
+      if (kFull || rel + 4 <= tn) __stcs(reinterpret_cast<float4*>(a.grad + q), make_float4(gr[0], gr[1], gr[2], gr[3]));
+      else
+        for (int c = 0; rel + c < tn; ++c) a.grad[q + c] = gr[c];
+    }
+  }
+}
 
 template <bool kSplit, bool kKL>
 __global__ void __launch_bounds__(kLossThreads, kKL ? 3 : 4) token_loss_kernel(LossArgs a, LossPlan lp) {
@@ -198,106 +358,19 @@ __global__ void __launch_bounds__(kLossThreads, kKL ? 3 : 4) token_loss_kernel(L
     return;
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float inv_t = a.inv_t;
+  LossWarp<kSplit, kKL>& ws = sm.warp[warp];
   // across tiles: float pairs for the policy term, the KL term and the sum of r (every
   // addition's rounding error kept in the low word), an integer count of clipped tokens
   float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   long long nclip_all = 0;
   const int64_t ntiles = a.N > 0 ? lp.ntiles : 0;  // (a valid plan has no tokens without edges)
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t t0 = tile * kLossTile;
-    const int tn = (int)min((int64_t)kLossTile, a.T - t0);  // tokens of this tile
-    // this thread's token chunks first (streaming loads, all in flight together), then the
-    // tile's edges: the two memory latencies overlap
-    float x[kLossChunks][4], y[kLossChunks][4], z[kLossChunks][4];
-#pragma unroll
-    for (int k = 0; k < kLossChunks; ++k) {
-      const int rel = 4 * (tid + k * kLossThreads);
-      const int64_t q = t0 + rel;
-      if (rel + 4 <= tn) {
-        const float4 u = __ldcs(reinterpret_cast<const float4*>(a.logp + q));
-        const float4 v = __ldcs(reinterpret_cast<const float4*>(a.old_logp + q));
-        x[k][0] = u.x, x[k][1] = u.y, x[k][2] = u.z, x[k][3] = u.w;
-        y[k][0] = v.x, y[k][1] = v.y, y[k][2] = v.z, y[k][3] = v.w;
-        if (kKL) {
-          const float4 w4 = __ldcs(reinterpret_cast<const float4*>(a.ref_logp + q));
-          z[k][0] = w4.x, z[k][1] = w4.y, z[k][2] = w4.z, z[k][3] = w4.w;
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const bool in = rel + c < tn;
-          x[k][c] = in ? a.logp[q + c] : 0.f;
-          y[k][c] = in ? a.old_logp[q + c] : 0.f;
-          if (kKL) z[k][c] = in ? a.ref_logp[q + c] : 0.f;
-        }
-      }
-    }
-    // edges [e_lo, e_hi] hold the tile's tokens (each edge has >= 1 token: at most kLossTile)
-    const int e_lo = min(max(lp.tile_edge[tile], 0), a.N - 1);
-    const int e_hi = min(max(lp.tile_edge[tile + 1], e_lo), min(a.N - 1, e_lo + kLossTile - 1));
-    const int ne = e_hi - e_lo + 1;
-    __syncthreads();  // the previous tile's readers are done
-    for (int j = tid; j <= ne; j += kLossThreads) {
-      const int64_t st = lp.start[e_lo + j] - t0;
-      sm.start[j] = (int16_t)max(min(st, (int64_t)kLossTile), (int64_t)0);  // clamped to the tile
-      if (j < ne) {
-        const float w = a.norm_token ? inv_t : lp.w[e_lo + j];
-        sm.wa[j] = w * a.adv[e_lo + j];
-        if (kSplit) sm.we[j] = a.mask[e_lo + j] ? w * (a.lambda * a.eff[e_lo + j]) : 0.f;
-        if (kKL) sm.w[j] = w;
-      }
-    }
-    __syncthreads();
-    // the token -> edge map of the tile: warp w fills the spans of edges w, w + 8, ...
-    for (int j = warp; j < ne; j += kLossThreads / 32)
-      for (int t = sm.start[j] + lane; t < sm.start[j + 1]; t += 32) sm.map[t] = (uint16_t)j;
-    __syncthreads();
+  const int64_t nwarps = (int64_t)gridDim.x * kLossWarps;
+  for (int64_t tile = (int64_t)blockIdx.x * kLossWarps + warp; tile < ntiles; tile += nwarps) {
+    const int tn = (int)min((int64_t)kLossTile, a.T - tile * kLossTile);  // tokens of this tile
     float pg = 0.f, kl = 0.f, rs = 0.f;
     int nclip = 0;
-#pragma unroll
-    for (int k = 0; k < kLossChunks; ++k) {
-      const int rel = 4 * (tid + k * kLossThreads);  // first token of this chunk in the tile
-      if (rel >= tn) continue;
-      const uint2 m4 = *reinterpret_cast<const uint2*>(sm.map + rel);  // the 4 tokens' edges
-      const int jj[4] = {(int)(m4.x & 0xFFFFu), (int)(m4.x >> 16), (int)(m4.y & 0xFFFFu), (int)(m4.y >> 16)};
-      float gr[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const bool in = rel + c < tn;
-        const int j = in ? min(jj[c], ne - 1) : 0;  // tokens past the tile's end read edge 0
-        const float r = __expf(x[k][c] - y[k][c]);
-        const float rc = fminf(fmaxf(r, a.lo), a.hi);
-        float f, df;
-        const bool clipped = surrogate(r, rc, sm.wa[j], f, df);
-        if (kSplit) {
-          float f2, df2;
-          surrogate(r, rc, sm.we[j], f2, df2);
-          f += f2;
-          df += df2;
-        }
-        float g = -df;
-        if (kKL) {
-          float em1, k3;
-          kl_terms(z[k][c] - x[k][c], em1, k3);
-          const float w = sm.w[j];
-          kl = in ? fmaf(w, k3, kl) : kl;
-          g = fmaf(-a.beta * w, em1, g);  // beta w (1 - e^x)
-        }
-        if (in) {
-          pg += f;
-          rs += r;
-          nclip += clipped ? 1 : 0;
-        }
-        gr[c] = g;
-      }
-      if (a.grad) {
-        const int64_t q = t0 + rel;
-        if (rel + 4 <= tn) __stcs(reinterpret_cast<float4*>(a.grad + q), make_float4(gr[0], gr[1], gr[2], gr[3]));
-        else
-          for (int c = 0; rel + c < tn; ++c) a.grad[q + c] = gr[c];
-      }
-    }
+    if (tn == kLossTile) tile_loss<kSplit, kKL, true>(a, lp, ws, tile, tn, lane, pg, kl, rs, nclip);
+    else tile_loss<kSplit, kKL, false>(a, lp, ws, tile, tn, lane, pg, kl, rs, nclip);
     ff_acc(acc[0].x, acc[0].y, pg);
     ff_acc(acc[1].x, acc[1].y, kl);
     ff_acc(acc[2].x, acc[2].y, rs);
@@ -404,7 +477,7 @@ cudaError_t launch_loss_variant(const LaunchCtx& lc, const LossPlan& lp, const L
   const int bytes = (int)sizeof(LossSmem<kSplit, kKL>);
   const int per_sm = kKL ? 3 : 4;  // resident CTAs (registers, shared memory)
   const int64_t cap = min((int64_t)lc.num_sms * per_sm, (int64_t)kLossMaxBlocks);
-  const int grid = (int)max((int64_t)1, min(lp.ntiles, cap));
+  const int grid = (int)max((int64_t)1, min((lp.ntiles + kLossWarps - 1) / kLossWarps, cap));
   token_loss_kernel<kSplit, kKL><<<grid, kLossThreads, bytes, lc.stream>>>(a, lp);
   return cudaGetLastError();
 }
