@@ -364,6 +364,7 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   pp.b_next = bud ? bud->b_next : 0;
   pp.active = bud ? bud->active : nullptr;
   pp.budget = bud ? bud->budget : nullptr;
+  pp.rest_stats = 0;
   pp.debug_timeout = (p.flags & GPO_FLAG_DEBUG_TIMEOUT) != 0;
   Ws ws = workspace_views(workspace, L);
   LaunchCtx lc;
@@ -423,6 +424,16 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   } else if (fused32) {
     if (e == cudaSuccess) e = stage("fused_f32", [&] { return launch_fused_f32(lc, b, *out, sz, ws, pp); });
   } else if (fused) {
+    // rows of d <= kRestStatsD: the statistics of the groups after each CTA's first by a launch
+    // on the whole GPU first, a few us that group_eta_stats' steps would cost every group (512
+    // groups of 320 states: d = 64 138 against 151 us, 256 162 / 167, 512 201 / 189, 1024 277 / 257)
+    const int grid = fused_grid(lc, sz);
+    if (e == cudaSuccess && !bud && sz.d <= kRestStatsD && g1 - g0 > (int64_t)grid) {
+      pp.rest_stats = 1;
+      Sizes rest = sz;
+      rest.g0 = sz.g0 + grid;
+      e = stage("exact_stats", [&] { return launch_exact_stats(lc, b, rest, ws); });
+    }
     if (e == cudaSuccess) e = stage("fused", [&] { return launch_fused(lc, map, map32, b, *out, sz, ws, pp); });
   } else {
     if (e == cudaSuccess && b.parent) e = stage("tree_prep", [&] { return launch_tree_prep(lc, b, sz, ws); });
@@ -432,7 +443,7 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
       // compensated statistics (fp32 embeddings, first then) or from row_stats; bf16 embeddings'
       // statistics follow the similarity stage or row_stats, whose norms give their sums' biases
       const bool exact_first = !use_tc && !bud && b.emb_dtype == GPO_EMB_F32;
-      auto exact = [&] { return launch_exact_stats(lc, b, sz, ws); };
+      auto exact = [&] { return launch_exact_stats(lc, b, sz, ws, true); };
       if (exact_first) e = stage("exact_stats", exact);
       else if (!use_tc) e = stage("row_stats", [&] { return launch_row_stats(lc, b, sz, ws); });
       if (e == cudaSuccess)

@@ -20,8 +20,9 @@
 //                   cos = acc / (|z_i||z_j|) >= kappa goes to an edge list; the
 //                   accumulator is released and the listed pairs are united in a
 //                   shared-memory union-find forest (Alg. S.1)
-//   warps 2..       per-group validation; once the classes are known, the compensated row
-//                   statistics of the rows whose eta(p(v), v) can reach a result, from L2;
+//   warps 2..       per-group validation; the compensated row statistics that eta(p(v), v)
+//                   needs: of every row while the group streams in (a CTA's first group), or,
+//                   once the classes are known, of the rows whose eta can reach a result;
 //                   graph reward and dual-group advantage (gpo_group_math.cuh) and the
 //                   token scatter (Sec. 4.5), overlapping the next group's loads and MMAs
 // Group ranges are assigned round-robin to CTAs.  Every wait is bounded.
@@ -56,12 +57,17 @@ cudaError_t setup_fused() {
   return e;
 }
 
+int fused_grid(const LaunchCtx& lc, const Sizes& sz) {
+  const int ng = sz.g1 - sz.g0;
+  const int cap = lc.num_sms * (sz.maxn <= fused_small::kMaxN ? fused_small::kMinBlocks : fused_large::kMinBlocks);
+  return ng < cap ? ng : cap;
+}
+
 cudaError_t launch_fused(const LaunchCtx& lc, const CUtensorMap& map, const CUtensorMap& map32, const gpo_batch& b,
                          const gpo_outputs& o, const Sizes& sz, const Ws& ws, const Params& p) {
   const int ng = sz.g1 - sz.g0;
   if (ng <= 0) return cudaSuccess;
-  const int cap = lc.num_sms * (sz.maxn <= fused_small::kMaxN ? fused_small::kMinBlocks : fused_large::kMinBlocks);
-  const int grid = ng < cap ? ng : cap;
+  const int grid = fused_grid(lc, sz);
   if (sz.maxn <= fused_small::kMaxN)
     fused_small::fused_kernel<<<grid, fused_small::kThreads, fused_small::fused_smem(), lc.stream>>>(map, map32, b, o,
                                                                                                    sz, ws, p);

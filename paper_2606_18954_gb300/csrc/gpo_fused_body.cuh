@@ -17,6 +17,7 @@ constexpr int kWarpEdges = 256;                 // linked pairs listed per epilo
 constexpr int kEdgeList = kWarpEdges * (kEpiThreads / 32);
 constexpr int kBarGroup = 1;                    // named barrier of the group warps
 constexpr int kBarEpi = 2;                      // named barrier of the drain warps
+constexpr int kBarSetup = 3;                    // named barrier of warps 2 and 3 (early set-up)
 static_assert(kThreads % 128 == 0 && kThreads >= 256 && kGThreads >= kMaxN, "fused kernel shape");
 
 struct Seg {
@@ -160,6 +161,7 @@ static_assert(kTilesOff + 1023 + kRingBytes <= 232448, "fused kernel exceeds 227
 
 __device__ __forceinline__ void bar_group() { asm volatile("bar.sync %0, %1;" ::"n"(kBarGroup), "n"(kGThreads) : "memory"); }
 __device__ __forceinline__ void bar_epi() { asm volatile("bar.sync %0, %1;" ::"n"(kBarEpi), "n"(kEpiThreads) : "memory"); }
+__device__ __forceinline__ void bar_setup() { asm volatile("bar.sync %0, %1;" ::"n"(kBarSetup), "n"(64) : "memory"); }
 
 // Bits a..31 of a word (all for a <= 0, none for a >= 32).
 __device__ __forceinline__ uint32_t bits_from(int a) { return a <= 0 ? 0xFFFFFFFFu : (a >= 32 ? 0u : 0xFFFFFFFFu << a); }
@@ -186,8 +188,8 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
   return v;
 }
 
-// The compensated row statistics that the group's eta's ask for (every group but the first
-// of a CTA in a branching batch, see group_row_stats; all group threads, one
+// The compensated row statistics that the group's eta's ask for (where group_row_stats has
+// not computed every row's; all group threads, one
 // state each: thread gt has state gt; need: eta(p(v), v) of that state is read).  The rows
 // are known only once the classes are, when they have just been streamed and lie in L2, and
 // they are few: 0.2 to 0.45 of a chain batch's states (a step whose score differs from its
@@ -255,18 +257,27 @@ __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes&
   bar_group();
 }
 
-// Compensated |z_v|^2 and <z_{p(v)}, z_v> of every state of a branching group into ws.x_n2 /
-// ws.x_dot (float pairs), by the group warps while the producer streams the same rows: for
-// a CTA's first group, when they would otherwise wait for the stream.  A branching batch
-// reads 0.85 of its eta's, so little of it is in vain (tree: 71.0 us, against 74.4 us with
-// group_eta_stats in its place; a chain batch reads a third of them, and there the rows of
-// group_eta_stats after the classes are the better: math 58.0 against 58.7 us, agentic
-// with all outputs 54.9 against 57.9).  The warps claim blocks of 8 rows; lane 4 r + c takes
-// every fourth 16-byte chunk of row r from chunk c; a parent that is the row before comes
-// from the lane 4 below.  bf16 products are exact in fp32, sums by TwoSum (no bound of the
-// norms is known yet), the row's 4 partial pairs combined in a fixed butterfly.
+// Compensated |z_v|^2 and <z_{p(v)}, z_v> of every state of a group into ws.x_n2 / ws.x_dot
+// (float pairs), by the group warps while the producer streams the same rows: for a CTA's
+// first group, when they would otherwise wait for the stream, of a branching batch or with
+// rows of d < kEarlyD.  All rows' statistics then take no longer than the stream and what
+// follows it, while group_eta_stats is a serial step after the classes; with wider rows its
+// third of a chain batch's rows is the less (128 groups of 256 states, us, these statistics
+// against group_eta_stats: d = 64 31.4 / 39.6, 256 37.9 / 43.6, 512 43.7 / 45.8, 768 60.0 /
+// 60.1, 1024 60.0 / 58.0, 2048 111 / 95; 256 groups of 56: d = 256 27.2 / 33.4, 768 34.4 / 37.5,
+// 1024 39.5 / 39.6, 2048 58.0 / 51.9).  A branching batch reads 0.85 of its eta's (tree, d =
+// 1024: 71.0 / 74.4).  The calling warps claim blocks of 8 rows from gs->nstat[0] until none is
+// left, so that warps that join late or run slower take fewer; lane 4 r + c takes every fourth
+// 16-byte chunk of row r from chunk c; a parent that is the row before comes from the lane 4
+// below, other parents and the prompt embedding are loaded.  Parents: with `early` (chain
+// layout, before the group's set-up) the previous state for every state but the group's first
+// (the set-up fixes the rollouts' first states afterwards: their parent is the prompt root);
+// otherwise from the group layout in shared memory.  bf16 products are exact in fp32, sums by
+// TwoSum (no bound of the norms is known yet), the row's 4 partial pairs combined in a fixed
+// butterfly.
+constexpr int kEarlyD = 1024;
 __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
-                                                int g, int s0, int n, int lane, uint32_t* st) {
+                                                int g, int s0, int n, bool tree, bool early, int lane, uint32_t* st) {
   const int r = lane >> 2, c = lane & 3;
   const int nch = sz.d / 8;          // whole 16-byte chunks of a row
   const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
@@ -280,10 +291,15 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
   for (int blk = claim(); blk * 8 < n; blk = claim()) {
     const int i = blk * 8 + r;  // local row of this lane
     const bool live = i < n;
-    int pl = -1;  // parent: >= 0 a local row, -2 the prompt embedding, -1 none (eta 0)
+    // parent: >= 0 a local row, -2 the prompt embedding, -1 none (eta 0)
+    int pl = -1;
     if (live) {
-      pl = gs->par[i];
-      if (pl < 0) pl = b.root_emb ? -2 : -1;
+      if (early) {
+        pl = i - 1;
+      } else {
+        pl = tree ? gs->par[i] : (gs->dep[i] > 1 ? i - 1 : -1);
+        if (pl < 0) pl = b.root_emb ? -2 : -1;
+      }
     }
     const bool from_left = pl >= 0 && pl == i - 1 && r > 0;
     // (debug build) the rows this lane reads; the whole warp skips the block if any is out of
@@ -294,7 +310,8 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
     const uint4* zb = Z + (int64_t)(s0 + (live ? i : 0)) * rs;
     const uint4* pb = pl >= 0 ? Z + (int64_t)(s0 + pl) * rs : (pl == -2 ? RZ + (int64_t)g * rs : nullptr);
     uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
-    // two stages of kU chunks per lane, software-pipelined
+    // two stages of kU chunks per lane, software-pipelined: the next stage's loads are in
+    // flight while this one's sums run (no register copies between the stages)
     constexpr int kU = 2;
     auto load = [&](int k0, uint4 (&x)[kU], uint4 (&y)[kU]) {
 #pragma unroll
@@ -305,7 +322,7 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
         y[u] = !from_left && pb && in ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
       }
     };
-    auto accumulate = [&](const uint4 (&x)[kU], uint4 (&y)[kU]) {
+    auto accumulate = [&](uint4 (&x)[kU], uint4 (&y)[kU]) {
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         uint4 t;
@@ -318,7 +335,7 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
           const uint64_t xx = bf16x2_f32x2(xw[h]), yy = bf16x2_f32x2(yw[h]);
-          f2_acc(ns, ne, f2mul(xx, xx));
+          f2_acc(ns, ne, f2mul(xx, xx));  // bf16 products are exact in fp32
           f2_acc(ds, de, f2mul(xx, yy));
         }
       }
@@ -341,10 +358,12 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
         f2_acc(ds, de, f2mul(xx, pack_f2(pr ? (uint32_t)pr[k] << 16 : 0u, 0u)));
       }
     }
-    const float2 n2 = lanes_pair_sum<4>(f2_finish(ns, ne)), dot = lanes_pair_sum<4>(f2_finish(ds, de));
+    const float2 n2 = lanes_pair_sum<4>(f2_finish(ns, ne));
+    float2 dot = lanes_pair_sum<4>(f2_finish(ds, de));
+    if (pl == -1) dot = make_float2(0.f, 0.f);
     if (live && c == 0 && GPO_BOUNDS(st, s0 + i, sz.N, kWhereStats)) {
       ws.x_n2[s0 + i] = n2;
-      ws.x_dot[s0 + i] = pl == -1 ? make_float2(0.f, 0.f) : dot;
+      ws.x_dot[s0 + i] = dot;
     }
   }
 }
@@ -486,6 +505,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     mbar_init(&ctl->tempty, kEpiThreads / 32);
     mbar_init(&ctl->drain, 1);
     fence_mbar_init();
+    gs->nstat[0] = gs->nstat[1] = 0;
     tma_prefetch_desc(&zmap);
     tma_prefetch_desc(&zmap32);
   }
@@ -645,14 +665,29 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         make_plan(n, gs->plan);
         gs->flags = 0;
         gs->overflow = 0;
-        gs->nstat[0] = gs->nstat[1] = 0;
       }
+
+      // ---- compensated row statistics of every row (group_row_stats), for a CTA's first group
+      //      where they pay.  Chain layout without prompt embeddings: the drain warps start at
+      //      once (every state's parent taken as the state before it; a rollout's first state
+      //      then has eta 0 whatever its dot) while warps 2 and 3 lay out the group, then
+      //      join them; otherwise all group warps after the set-up.
+      const bool first = g < sz.g0 + (int)gridDim.x;
+      const bool stats_here = p.mode == 0 && (tree || sz.d < kEarlyD) && first;
+      const bool early = stats_here && !tree && b.root_emb == nullptr;
+      if (early && epi) group_row_stats(b, sz, ws, gs, g, s0, n, false, true, lane, st);
+
 
       if (tree) {
         tree_setup(b, sz, gs, g, r0, nr, s0, n, gt, wg, lane, st);
-      } else {
-      // ---- validate the group and lay out its states (Sec. 4.2 chain layout)
-      const int tid = gt, nt = kGThreads;
+      } else if (!early || !epi) {
+      // ---- validate the group and lay out its states (Sec. 4.2 chain layout): all group
+      //      threads, or warps 2 and 3 alone while the drain warps read the statistics
+      const int tid = gt, nt = early ? 64 : kGThreads;  // warps 2 and 3: gt = 0..63
+      auto sync = [&] {
+        if (early) bar_setup();
+        else bar_group();
+      };
       for (int r = tid; r <= nr; r += nt) {
         gs->rstart[r] = b.rollout_step_off[r0 + r] - s0;
         gs->tok0[r] = b.rollout_token_off[r0 + r];
@@ -666,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         gs->dep[i] = 1;
         gs->eadv[i] = 0.f;  // (the marks of group_eta_stats)
       }
-      bar_group();
+      sync();
       for (int r = tid; r < nr; r += nt) {
         const int a = gs->rstart[r], e = gs->rstart[r + 1];
         bool bad = !(a >= 0 && e > a && e <= n) || gs->rew[r] > 1;
@@ -688,17 +723,30 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           atomicOr(&gs->flags, 1);
         }
       }
+      if (early) group_row_stats(b, sz, ws, gs, g, s0, n, false, true, lane, st);  // join the drain warps
       }
-      bar_group();  // set-up complete
+      bar_group();  // set-up (and with `early` the row statistics) complete
       const bool valid = (gs->flags & 1) == 0;
-      const bool early = tree && p.mode == 0 && g < sz.g0 + (int)gridDim.x;  // the CTA's first group
-      if (early && valid) group_row_stats(b, sz, ws, gs, g, s0, n, lane, st);
+      if (!early && valid && stats_here) group_row_stats(b, sz, ws, gs, g, s0, n, tree, false, lane, st);
       if (valid && p.mode == 0 && b.root_emb && wg == 0) {  // |prompt embedding|^2, one warp
         float2 n2, dot;
         exact_pair_sums<true>(b.root_emb, (int64_t)g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
         if (lane == 0) {
           if (!isfinite(n2.x)) report(st, GPO_ERR_NONFINITE, 3, sz.N + g);
           ws.x_root_n2[g] = n2;
+        }
+      }
+
+      // ---- eta(p(v), v) of every state from the finished statistics, by warps 2 and 3 while
+      //      the drain warps test the pairs (with `early`: no prompt embedding, a rollout's
+      //      first state has eta 0); the group math takes it from ecor / eeff, which it
+      //      overwrites only with its own outputs, state by state, after reading it
+      if (early && valid && !epi) {
+        for (int i = gt; i < n; i += 64) {
+          const float2 e = gs->dep[i] == 1 ? make_float2(0.f, 0.f)
+                                           : ff_eta(ws.x_dot[s0 + i], ws.x_n2[s0 + i - 1], ws.x_n2[s0 + i]);
+          gs->ecor[i] = e.x;
+          gs->eeff[i] = e.y;
         }
       }
 
@@ -887,17 +935,19 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       }
       // ---- graph reward and dual-group advantage of every edge
       else if (valid) {
-        // eta(p(v), v) from the compensated row statistics: of every row (early), else of the
-        // rows that ask for it
+        // eta(p(v), v) from the compensated row statistics: of every row, in the workspace, or of
+        // the rows that ask for it
+        const bool all_rows = stats_here || (!first && p.rest_stats);
         auto par = [&](int i) { return tree ? gs->par[i] : (gs->dep[i] == 1 ? -1 : i - 1); };
         auto etas = [&](const bool (&need)[1]) {
-          if (!early) group_eta_stats(b, sz, ws, gs, g, s0, n, need[0], par, gt, wg, lane, st);
+          if (!all_rows) group_eta_stats(b, sz, ws, gs, g, s0, n, need[0], par, gt, wg, lane, st);
         };
         auto eta = [&](int i) -> float2 {
+          if (early) return make_float2(gs->ecor[i], gs->eeff[i]);
           const int q = par(i);  // -1: the prompt embedding
-          const float2 nq = q < 0 ? ws.x_root_n2[g] : (early ? ws.x_n2[s0 + q] : make_float2(gs->rn[q], gs->thr[q]));
-          return early ? ff_eta(ws.x_dot[s0 + i], nq, ws.x_n2[s0 + i])
-                       : ff_eta(make_float2(gs->ecor[i], gs->eeff[i]), nq, make_float2(gs->rn[i], gs->thr[i]));
+          const float2 nq = q < 0 ? ws.x_root_n2[g] : (all_rows ? ws.x_n2[s0 + q] : make_float2(gs->rn[q], gs->thr[q]));
+          return all_rows ? ff_eta(ws.x_dot[s0 + i], nq, ws.x_n2[s0 + i])
+                          : ff_eta(make_float2(gs->ecor[i], gs->eeff[i]), nq, make_float2(gs->rn[i], gs->thr[i]));
         };
         const bool has_root = b.root_emb != nullptr;
         auto out = [&](int i, int label, float S, float acor, float E, float dual, unsigned char mask) {
@@ -975,6 +1025,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           }
         }
       }
+      if (gt == 0) gs->nstat[0] = gs->nstat[1] = 0;  // for the next group
       bar_group();
     }
   }

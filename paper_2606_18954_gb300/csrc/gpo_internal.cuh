@@ -20,6 +20,7 @@ constexpr int kEdgeCap = 384;        // spanning-forest edges one item can emit 
 constexpr int kStatusWords = 16;
 constexpr int kMaxStages = 8;        // timed stages of one gpo_compute
 constexpr int kFusedMaxStates = 384; // largest group of the fused group-resident kernel
+constexpr int kRestStatsD = 256;     // widest rows whose statistics a launch before the fused kernel computes
 constexpr int kPipeMaxChunks = 64;   // gpo_compute_host: pipeline stages at most
 constexpr int kPipeComputeStreams = 3;
 constexpr int64_t kPipeMinChunkBytes = (int64_t)8 << 20;
@@ -93,6 +94,8 @@ struct Params {
   int ddof, rule;
   // mode 1: next-layer budgets after layer `layer` instead of advantages (gpo_layer_budget)
   int mode, layer, b_next;
+  int rest_stats;         // fused path: exact_stats has computed the compensated row statistics of
+                          // the groups after each CTA's first
   int debug_timeout;      // GPO_FLAG_DEBUG_TIMEOUT: the MMA warp's first wait runs out
   const uint8_t* active;  // [N] frontier states to expand (NULL: all of depth `layer`)
   int32_t* budget;        // [N] output of mode 1
@@ -484,8 +487,8 @@ __device__ __forceinline__ float2 f2_finish(uint64_t s, uint64_t e) {
 //   t = fma(x, y, s),  z = s - t,  err = fma(x, y, z) = p - (t - s)
 // gives the rounding error of every addition exactly (collected, rounded, in e).  s - sigma
 // is exact (Sterbenz), so the sum is (s - sigma) + e.  B comes from the similarity stage's
-// fp32 squared norms (|x y| <= (x^2 + y^2) / 2 for a dot): sigma = 2^ceil(log2 (4.04 |x|^2))
-// and 2^ceil(log2 (2.02 (|x|^2 + |y|^2))).  Two fp32 lanes per instruction, as in f2_acc.
+// fp32 squared norms (Cauchy-Schwarz for a dot): sigma = 2^ceil(log2 (4.04 |x|^2)) and
+// 2^ceil(log2 (4.04 |x| |y|)).  Two fp32 lanes per instruction, as in f2_acc.
 
 __device__ __forceinline__ uint64_t f2fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
@@ -561,7 +564,7 @@ __device__ __forceinline__ void half_warp_row_sums(const uint4* x, const uint4* 
   const int nch = d / 8;
   BiasedSum sn, sd;
   bs_init(sn, pow2_ceil(4.04f * nx));
-  if (kDot) bs_init(sd, pow2_ceil(2.02f * (nx + ny)));
+  if (kDot) bs_init(sd, pow2_ceil(4.04f * (sqrtf(nx) * sqrtf(ny))));
   constexpr int kU = 2;  // chunks of a stage
   auto load = [&](int k0, uint4 (&a)[kU], uint4 (&b)[kU]) {
 #pragma unroll
@@ -754,8 +757,9 @@ struct LaunchCtx {
 };
 
 cudaError_t launch_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
-// (ws.nrm2 holds every row's fp32 squared norm)
-cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
+// with_norms: ws.nrm2 holds every row's fp32 squared norm (the similarity stage ran first)
+cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
+                               bool with_norms = false);
 cudaError_t launch_tree_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
 cudaError_t setup_tree_prep();
 cudaError_t launch_row_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
@@ -771,6 +775,8 @@ cudaError_t launch_tokens(const LaunchCtx& lc, const gpo_batch& b, const gpo_out
 // Records a message on the context (gpo_last_error).
 void note_error(gpo_ctx* ctx, const char* msg);
 
+// CTAs the fused kernel runs with for groups [g0, g1) (one group each when ng <= this).
+int fused_grid(const LaunchCtx& lc, const Sizes& sz);
 cudaError_t launch_fused(const LaunchCtx& lc, const CUtensorMap& map, const CUtensorMap& map32, const gpo_batch& b,
                          const gpo_outputs& o, const Sizes& sz, const Ws& ws, const Params& p);
 cudaError_t setup_fused();

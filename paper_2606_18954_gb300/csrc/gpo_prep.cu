@@ -476,8 +476,25 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const bool tree = b.parent != nullptr;
-  const int64_t jobs = (int64_t)sz.N + (b.root_emb ? sz.G : 0);  // the states, then the prompt embeddings
-  for (int64_t job = warp; job < jobs; job += nwarps) {
+  // the states and prompt embeddings of groups [g0, g1) (the whole batch, or the groups after the
+  // fused kernel's first ones)
+  int v0 = 0, v1 = sz.N;
+  if (sz.g0 != 0 || sz.g1 != sz.G) {
+    const int32_t* go = b.group_rollout_off;
+    if (tree) {
+      v0 = b.group_state_off[sz.g0];
+      v1 = b.group_state_off[sz.g1];
+    } else {
+      const int ra = go[sz.g0], rb = go[sz.g1];
+      v0 = ra >= 0 && ra <= sz.R ? b.rollout_step_off[ra] : 0;
+      v1 = rb >= 0 && rb <= sz.R ? b.rollout_step_off[rb] : 0;
+    }
+    v0 = max(0, min(v0, sz.N));
+    v1 = max(v0, min(v1, sz.N));
+  }
+  const int nstate = v1 - v0, nroot = b.root_emb ? sz.g1 - sz.g0 : 0;
+  for (int64_t jj = warp; jj < (int64_t)nstate + nroot; jj += nwarps) {
+    const int64_t job = jj < nstate ? v0 + jj : sz.N + sz.g0 + (jj - nstate);
     if (job >= sz.N) {  // |prompt embedding|^2
       const int64_t g = job - sz.N;
       float2 n2, dot;
@@ -524,11 +541,17 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
 // holds (a shuffle); the first row's parent chunk, a tree parent or a prompt embedding is
 // loaded.  Compensated sums per lane, two fp32 lanes per instruction, then a fixed butterfly
 // over the 4 quarters: the accuracy of exact_stats_kernel with every row read once.
-// The similarity stage (or row_stats) has left fp32 squared norms in ws.nrm2, accurate to
-// far better than 1 %: the biases of error-free biased sums (BiasedSum), four fp32
-// operations per product, two independent chains per sum.  A lane whose sum ends outside
-// its range (a norm that was not what it was taken for) sends its row through TwoSum per
-// product instead.
+//   kNorms = false (before the fused kernel, for the groups after its CTAs' first): TwoSum per
+//   product (f2_acc).
+//   kNorms = true (after the similarity stage, which leaves fp32 squared norms in ws.nrm2,
+//   accurate to far better than 1 %): biased error-free sums with one bias per row and sum,
+//   sigma = 2^ceil(log2 (4.04 |z_v|^2)) for |z_v|^2 and 2^ceil(log2 (2.02 (|z_v|^2 + |z_p|^2)))
+//   for <z_p, z_v> (|x y| <= (x^2 + y^2) / 2), so that each running sum stays in
+//   [sigma/2, 3 sigma/2] and every product is Fast2Sum's case (see BiasedSum): four fp32
+//   operations per product, two independent chains per sum, no bound pass.  A lane whose sum
+//   ends outside the range (a norm that was not what the similarity stage reported) sends its
+//   row through the TwoSum path instead.
+template <bool kNorms>
 __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Sizes sz, Ws ws) {
   const int lane = threadIdx.x & 31, r = lane >> 2, j = lane & 3;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -538,6 +561,33 @@ __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Size
   const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
   const uint4* Z = reinterpret_cast<const uint4*>(b.emb);
   const uint4* RZ = reinterpret_cast<const uint4*>(b.root_emb);
+  int v0 = 0, v1 = sz.N;  // states of groups [g0, g1)
+  if (sz.g0 != 0 || sz.g1 != sz.G) {
+    if (tree) {
+      v0 = b.group_state_off[sz.g0];
+      v1 = b.group_state_off[sz.g1];
+    } else {
+      const int ra = b.group_rollout_off[sz.g0], rb = b.group_rollout_off[sz.g1];
+      v0 = ra >= 0 && ra <= sz.R ? b.rollout_step_off[ra] : 0;
+      v1 = rb >= 0 && rb <= sz.R ? b.rollout_step_off[rb] : 0;
+    }
+    v0 = max(0, min(v0, sz.N));
+    v1 = max(v0, min(v1, sz.N));
+  }
+  auto quad = [&](float2 P) -> float2 {  // the 4 quarters' pairs, fixed order
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      const float a = __shfl_xor_sync(0xffffffffu, P.x, o), c = __shfl_xor_sync(0xffffffffu, P.y, o);
+      float t, u;
+      two_sum(P.x, a, t, u);
+      P.x = t;
+      P.y = P.y + c + u;
+    }
+    float h, l;
+    two_sum(P.x, P.y, h, l);
+    return make_float2(h, l);
+  };
+  auto finish4 = [&](uint64_t s, uint64_t e) -> float2 { return quad(f2_finish(s, e)); };
   // TwoSum sums of this lane's quarter of row zb and its parent pb (chunks loaded here)
   auto twosum_quarter = [&](const uint4* zb, const uint4* pb, bool on, float2& n2, float2& dot) {
     uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
@@ -552,11 +602,10 @@ __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Size
         f2_acc(ds, de, f2mul(xx, yy));
       }
     }
-    n2 = lanes_pair_sum<4>(f2_finish(ns, ne));
-    dot = lanes_pair_sum<4>(f2_finish(ds, de));
+    n2 = finish4(ns, ne);
+    dot = finish4(ds, de);
   };
-  const int v1 = sz.N;
-  for (int64_t base = warp * 8; base < v1; base += nwarps * 8) {
+  for (int64_t base = v0 + warp * 8; base < v1; base += nwarps * 8) {
     const int64_t v = base + r;
     const bool live = v < v1;
     // the rollout (chain) or group (tree) of the warp's first row by a 32-ary search, then each
@@ -599,59 +648,104 @@ __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Size
     const uint4* pb = p >= 0 ? Z + (int64_t)p * rs : (p <= -2 ? RZ + (int64_t)(-2 - p) * rs : nullptr);
     const uint4* zb = Z + (live ? v : base) * rs;
     float2 n2, dot;
-    // the biases: fp32 squared norms of the row and its parent (ws.nrm2; the prompt
-    // embedding's from root_norms_kernel, which ran first)
-    float nv = 0.f, np = 0.f;
-    if (live) {
-      nv = ws.nrm2[v];
-      if (p >= 0) np = ws.nrm2[p];
-      else if (p <= -2) np = ws.x_root_n2[-2 - p].x;
-    }
-    BiasedSum sn, sd;
-    bs_init(sn, pow2_ceil(4.04f * nv));
-    bs_init(sd, pow2_ceil(2.02f * (nv + np)));
-    constexpr int kU = 4;  // chunks loaded ahead of their arithmetic (memory-level parallelism)
-    for (int c0 = 0; c0 < nq; c0 += kU) {
-      uint4 x[kU], y[kU];
+    if (!kNorms) {
+      uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
+      constexpr int kU = 4;  // chunks loaded ahead of their arithmetic (memory-level parallelism)
+      for (int c0 = 0; c0 < nq; c0 += kU) {
+        uint4 x[kU], y[kU];
 #pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int k = j * nq + c0 + u;
-        x[u] = live && c0 + u < nq ? zb[k] : make_uint4(0u, 0u, 0u, 0u);
-        y[u] = (!from_left && pb && c0 + u < nq) ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
-      }
+        for (int u = 0; u < kU; ++u) {
+          const int k = j * nq + c0 + u;
+          x[u] = live && c0 + u < nq ? zb[k] : make_uint4(0u, 0u, 0u, 0u);
+          y[u] = (!from_left && pb && c0 + u < nq) ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
+        }
 #pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        uint4 t;
-        t.x = __shfl_up_sync(0xffffffffu, x[u].x, 4);
-        t.y = __shfl_up_sync(0xffffffffu, x[u].y, 4);
-        t.z = __shfl_up_sync(0xffffffffu, x[u].z, 4);
-        t.w = __shfl_up_sync(0xffffffffu, x[u].w, 4);
-        if (from_left) y[u] = t;
-        const uint32_t xw[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yw[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+        for (int u = 0; u < kU; ++u) {
+          uint4 t;
+          t.x = __shfl_up_sync(0xffffffffu, x[u].x, 4);
+          t.y = __shfl_up_sync(0xffffffffu, x[u].y, 4);
+          t.z = __shfl_up_sync(0xffffffffu, x[u].z, 4);
+          t.w = __shfl_up_sync(0xffffffffu, x[u].w, 4);
+          if (from_left) y[u] = t;
+          const uint32_t xw[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yw[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
 #pragma unroll
-        for (int h = 0; h < 4; h += 2) {
-          const uint64_t x0 = bf16x2_f32x2(xw[h]), y0 = bf16x2_f32x2(yw[h]);
-          const uint64_t x1 = bf16x2_f32x2(xw[h + 1]), y1 = bf16x2_f32x2(yw[h + 1]);
-          biased_add(sn.s0, sn.e0, x0, x0);
-          biased_add(sd.s0, sd.e0, x0, y0);
-          biased_add(sn.s1, sn.e1, x1, x1);
-          biased_add(sd.s1, sd.e1, x1, y1);
+          for (int h = 0; h < 4; ++h) {
+            const uint64_t xx = bf16x2_f32x2(xw[h]), yy = bf16x2_f32x2(yw[h]);
+            f2_acc(ns, ne, f2mul(xx, xx));  // bf16 products are exact in fp32
+            f2_acc(ds, de, f2mul(xx, yy));
+          }
         }
       }
-    }
-    int okv = !live || (bs_in_range(sn) && bs_in_range(sd));
-    // the row's 4 lanes agree (lanes 4 r .. 4 r + 3); every lane takes part in both shuffles
-    okv &= __shfl_xor_sync(0xffffffffu, okv, 1);
-    okv &= __shfl_xor_sync(0xffffffffu, okv, 2);
-    const bool ok = okv != 0;
-    n2 = lanes_pair_sum<4>(bs_pair(sn));
-    dot = lanes_pair_sum<4>(bs_pair(sd));
-    if (__any_sync(0xffffffffu, !ok)) {  // rare: the rows out of range, by TwoSum
-      float2 n2b, dotb;
-      twosum_quarter(zb, pb, live && !ok, n2b, dotb);
-      if (!ok) {
-        n2 = n2b;
-        dot = dotb;
+      n2 = finish4(ns, ne);
+      dot = finish4(ds, de);
+    } else {
+      // the biases: fp32 squared norms of the row and its parent (ws.nrm2; the prompt
+      // embedding's from root_norms_kernel, which ran first)
+      float nv = 0.f, np = 0.f;
+      if (live) {
+        nv = ws.nrm2[v];
+        if (p >= 0) np = ws.nrm2[p];
+        else if (p <= -2) np = ws.x_root_n2[-2 - p].x;
+      }
+      const float sgn = pow2_ceil(4.04f * nv), sgd = pow2_ceil(2.02f * (nv + np));
+      const uint64_t sn0 = f2splat(sgn), sd0 = f2splat(sgd);
+      uint64_t a0 = sn0, a1 = sn0, b0 = sd0, b1 = sd0, ea0 = 0ull, ea1 = 0ull, eb0 = 0ull, eb1 = 0ull;
+      constexpr int kU = 4;
+      for (int c0 = 0; c0 < nq; c0 += kU) {
+        uint4 x[kU], y[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int k = j * nq + c0 + u;
+          x[u] = live && c0 + u < nq ? zb[k] : make_uint4(0u, 0u, 0u, 0u);
+          y[u] = (!from_left && pb && c0 + u < nq) ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          uint4 t;
+          t.x = __shfl_up_sync(0xffffffffu, x[u].x, 4);
+          t.y = __shfl_up_sync(0xffffffffu, x[u].y, 4);
+          t.z = __shfl_up_sync(0xffffffffu, x[u].z, 4);
+          t.w = __shfl_up_sync(0xffffffffu, x[u].w, 4);
+          if (from_left) y[u] = t;
+          const uint32_t xw[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yw[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+#pragma unroll
+          for (int h = 0; h < 4; h += 2) {
+            const uint64_t x0 = bf16x2_f32x2(xw[h]), y0 = bf16x2_f32x2(yw[h]);
+            const uint64_t x1 = bf16x2_f32x2(xw[h + 1]), y1 = bf16x2_f32x2(yw[h + 1]);
+            biased_add(a0, ea0, x0, x0);
+            biased_add(b0, eb0, x0, y0);
+            biased_add(a1, ea1, x1, x1);
+            biased_add(b1, eb1, x1, y1);
+          }
+        }
+      }
+      // every running sum still in [sigma/2, 3 sigma/2]: then each step was error-free
+      auto in_range = [](uint64_t s, float sg) {
+        uint32_t lo, hi;
+        unpack_f2(s, lo, hi);
+        return fabsf(__uint_as_float(lo) - sg) <= 0.5f * sg && fabsf(__uint_as_float(hi) - sg) <= 0.5f * sg;
+      };
+      int okv = !live || (in_range(a0, sgn) && in_range(a1, sgn) && in_range(b0, sgd) && in_range(b1, sgd));
+      // the row's 4 lanes agree (lanes 4 r .. 4 r + 3); every lane takes part in both shuffles
+      okv &= __shfl_xor_sync(0xffffffffu, okv, 1);
+      okv &= __shfl_xor_sync(0xffffffffu, okv, 2);
+      const bool ok = okv != 0;
+      // (s - sigma) is exact in each lane; the lane's pair: both chains' parts and errors
+      auto lane_pair = [](uint64_t s0, uint64_t e0, uint64_t s1, uint64_t e1, float sg) {
+        uint64_t h = 0ull, l = 0ull;
+        f2_acc(h, l, f2sub(s0, f2splat(sg)));
+        f2_acc(h, l, f2sub(s1, f2splat(sg)));
+        return f2_finish(h, f2add(l, f2add(e0, e1)));
+      };
+      n2 = quad(lane_pair(a0, ea0, a1, ea1, sgn));
+      dot = quad(lane_pair(b0, eb0, b1, eb1, sgd));
+      if (__any_sync(0xffffffffu, !ok)) {  // rare: the rows out of range, by TwoSum
+        float2 n2b, dotb;
+        twosum_quarter(zb, pb ? pb : nullptr, live && !ok, n2b, dotb);
+        if (!ok) {
+          n2 = n2b;
+          dot = dotb;
+        }
       }
     }
     if (p == -1) dot = make_float2(0.f, 0.f);
@@ -663,12 +757,12 @@ __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Size
   }
 }
 
-// |prompt embedding|^2, one warp each (exact_stats_lane_kernel covers the states).
+// |prompt embedding|^2 of groups [g0, g1), one warp each (the streamed kernel covers the states).
 __global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, Ws ws) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t g = warp; g < sz.G; g += nwarps) {
+  for (int64_t g = sz.g0 + warp; g < sz.g1; g += nwarps) {
     float2 n2, dot;
     exact_pair_sums<true>(b.root_emb, g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
     if (lane == 0) {
@@ -678,8 +772,9 @@ __global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, 
   }
 }
 
-cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws) {
-  const int64_t jobs = (int64_t)sz.N + (b.root_emb ? sz.G : 0);
+cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
+                               bool with_norms) {
+  const int64_t jobs = (int64_t)sz.N + (b.root_emb ? sz.G : 0);  // at most (range calls take fewer)
   if (jobs == 0) return cudaSuccess;
   const bool aligned16 = (reinterpret_cast<uintptr_t>(b.emb) & 15u) == 0 && sz.stride % 8 == 0 && sz.d % 8 == 0 &&
                          (!b.root_emb || (reinterpret_cast<uintptr_t>(b.root_emb) & 15u) == 0);
@@ -687,12 +782,15 @@ cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Si
     int64_t blocks = ((int64_t)sz.N + 63) / 64;  // a warp per 8 rows
     const int64_t bcap = (int64_t)lc.num_sms * 32;
     blocks = blocks < 1 ? 1 : (blocks > bcap ? bcap : blocks);
-    if (b.root_emb) {  // first: their norms enter the biases
-      int64_t rblocks = ((int64_t)sz.G + 7) / 8;
+    if (b.root_emb && sz.g1 > sz.g0) {  // first: the norms-based path reads them
+      int64_t rblocks = ((int64_t)(sz.g1 - sz.g0) + 7) / 8;
       if (rblocks > (int64_t)lc.num_sms * 8) rblocks = (int64_t)lc.num_sms * 8;
       root_norms_kernel<<<(int)rblocks, 256, 0, lc.stream>>>(b, sz, ws);
     }
-    exact_stats_lane_kernel<<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws);
+    if (with_norms)
+      exact_stats_lane_kernel<true><<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws);
+    else
+      exact_stats_lane_kernel<false><<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws);
     return cudaGetLastError();
   }
   int64_t blocks = (jobs + 7) / 8;  // a warp per row

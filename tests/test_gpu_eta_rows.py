@@ -1,10 +1,10 @@
-"""The group-resident bf16 kernel's compensated row statistics: computed only for the rows
-whose eta(p(v), v) can reach a result, by half-warps in stages of 64 chunks of 16 bytes, for
-every group of a chain batch and for the groups after a CTA's first of a branching one.
-More groups than CTAs (156 groups of more than 128 states), rows that are no multiple of a
-stage, of a half-warp or of a chunk, with and without prompt embeddings, and rows whose norms
-span many binades (each sum's bias comes from its row's own norm).  Same bar as the parity
-tests: class ids exact, |gpu - ref| <= 1e-5 |ref| + 1e-6."""
+"""The group-resident bf16 kernel's compensated row statistics: of every row while it streams in
+(a CTA's first group of a branching batch or with d < 1024), else of the rows whose eta(p(v), v)
+can reach a result, by half-warps in stages of 64 chunks of 16 bytes.  More groups than CTAs (156
+groups of more than 128 states), rows that are no multiple of a stage, of a half-warp or of a
+chunk, with and without prompt embeddings, and rows whose norms span many binades (each sum's
+bias comes from its rows' own norms).  Same bar as the
+parity tests: class ids exact, |gpu - ref| <= 1e-5 |ref| + 1e-6."""
 import dataclasses
 
 import numpy as np
