@@ -3,6 +3,7 @@
 //   prep (validate + plan) -> row stats -> similarity merge -> per-group
 //   advantages -> per-token scatter
 // all on the caller's stream.  Nothing here allocates device memory.
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -22,6 +23,8 @@ struct gpo_ctx {
   int num_sms;
   uint32_t* host_status;      // pinned copy of the workspace status words
   const uint32_t* last_status; // device status words of the last gpo_compute
+  uint64_t tag;                // tag of the errors of the calls since the last clearing one (see Status)
+  uint64_t last_tag;           // tag of last_status
   char msg[512];
   bool timing;
   int nstages;                 // stages recorded by the last gpo_compute
@@ -248,6 +251,7 @@ gpo_status gpo_create(gpo_ctx** out, const gpo_params* params) {
   if (!c) return GPO_ERR_CUDA;
   c->params = *params;
   c->last_status = nullptr;
+  c->tag = c->last_tag = kClearedTag;
   c->msg[0] = 0;
   cudaDeviceProp prop;
   if (cudaGetDevice(&c->device) != cudaSuccess || cudaGetDeviceProperties(&prop, c->device) != cudaSuccess) {
@@ -309,6 +313,20 @@ gpo_status gpo_workspace_size(const gpo_ctx* ctx, const gpo_batch* batch, size_t
 
 namespace {
 
+// A tag that no other call of this process has (48 bits, never 0 or kClearedTag): a counter
+// passed through the finaliser of SplitMix64 (Steele, Lea, Flood 2014), a bijection of 64 bits,
+// of which the top 48 are kept, so that small integers or text in memory never look like one.
+uint64_t fresh_tag() {
+  static std::atomic<uint64_t> calls{0};
+  while (true) {
+    uint64_t z = calls.fetch_add(1, std::memory_order_relaxed) * 0x9E3779B97F4A7C15ull + 0x2545F4914F6CDD1Dull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z = (z ^ (z >> 31)) >> 16;
+    if (z > kClearedTag) return z;
+  }
+}
+
 // Next-layer budget request of gpo_layer_budget (mode 1 of the kernels).
 struct BudgetReq {
   int layer, b_next;
@@ -316,10 +334,15 @@ struct BudgetReq {
   int32_t* budget;
 };
 
-// The path for groups [g0, g1) of the batch; clears the status words first if `clear`.
+// What a call does with the status words first: nothing (its errors join those of the calls
+// since the last clearing one), clear them, or, where that saves the clearing, take a tag of
+// its own (kFresh: a whole call, with no later ranges that another context might add).
+enum class StatusInit { kKeep, kClear, kFresh };
+
+// The path for groups [g0, g1) of the batch.
 // With `bud`, the classes and the next-layer budgets instead of the advantages.
 gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs* out, void* workspace,
-                        size_t workspace_bytes, int64_t g0, int64_t g1, bool clear, void* stream,
+                        size_t workspace_bytes, int64_t g0, int64_t g1, StatusInit init, void* stream,
                         const BudgetReq* bud = nullptr) {
   if (!ctx) return GPO_ERR_INVALID_ARG;
   ctx->msg[0] = 0;
@@ -418,7 +441,22 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   };
   cudaError_t e = cudaSuccess;
   if (ctx->timing) e = cudaEventRecord(ctx->ev[0], lc.stream);
-  if (e == cudaSuccess && clear) e = cudaMemsetAsync(ws.status, 0, sizeof(uint32_t) * kStatusWords, lc.stream);
+  // A fresh tag instead of a memset for the one-kernel paths (the tiled path's planning words
+  // start from zero), but not in a graph, whose replays would share it
+  if (init == StatusInit::kFresh) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (!(fused || fused32) || cudaStreamIsCapturing(lc.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();  // (the legacy stream beside a capture: the memset reports it)
+      init = StatusInit::kClear;
+    } else {
+      ctx->tag = fresh_tag();
+    }
+  }
+  if (init == StatusInit::kClear) {
+    ctx->tag = kClearedTag;
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws.status, 0, sizeof(uint32_t) * kStatusWords, lc.stream);
+  }
+  ws.tag = ctx->tag;
   if (g1 <= g0) {
     // nothing to compute (a call that only clears the status words)
   } else if (fused32) {
@@ -457,6 +495,7 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   }
   ctx->nstages = ns;
   ctx->last_status = ws.status;
+  ctx->last_tag = ws.tag;
   if (e != cudaSuccess) return set_msg(ctx, "launch failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
   return GPO_OK;
 }
@@ -468,7 +507,8 @@ extern "C" {
 gpo_status gpo_compute(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs* out, void* workspace,
                        size_t workspace_bytes, void* stream) {
   if (!ctx || !batch) return GPO_ERR_INVALID_ARG;
-  return compute_impl(ctx, batch, out, workspace, workspace_bytes, 0, batch->num_groups, true, stream);
+  return compute_impl(ctx, batch, out, workspace, workspace_bytes, 0, batch->num_groups, StatusInit::kFresh,
+                      stream);
 }
 
 gpo_status gpo_layer_budget(gpo_ctx* ctx, const gpo_batch* batch, int32_t layer, int32_t b_next, const uint8_t* active,
@@ -483,7 +523,8 @@ gpo_status gpo_layer_budget(gpo_ctx* ctx, const gpo_batch* batch, int32_t layer,
   memset(&o, 0, sizeof o);
   o.class_id = class_id;
   const BudgetReq req = {layer, b_next, active, budget};
-  return compute_impl(ctx, batch, &o, workspace, workspace_bytes, 0, batch->num_groups, true, stream, &req);
+  return compute_impl(ctx, batch, &o, workspace, workspace_bytes, 0, batch->num_groups, StatusInit::kFresh,
+                      stream, &req);
 }
 
 gpo_status gpo_compute_groups(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs* out, int64_t first_group,
@@ -495,7 +536,7 @@ gpo_status gpo_compute_groups(gpo_ctx* ctx, const gpo_batch* batch, const gpo_ou
     return set_msg(ctx, "group range [%lld, %lld) outside the batch's %lld groups", (long long)first_group,
                    (long long)(first_group + num_groups), (long long)batch->num_groups), GPO_ERR_INVALID_ARG;
   return compute_impl(ctx, batch, out, workspace, workspace_bytes, first_group, first_group + num_groups,
-                      clear_status != 0, stream);
+                      clear_status != 0 ? StatusInit::kClear : StatusInit::kKeep, stream);
 }
 
 gpo_status gpo_compute_host(gpo_ctx* ctx, const gpo_batch* host, const gpo_batch* dev, const gpo_outputs* out,
@@ -584,7 +625,7 @@ gpo_status gpo_compute_host(gpo_ctx* ctx, const gpo_batch* host, const gpo_batch
   if (!piped) {  // one upload, the whole path, one download
     up(d.emb, h.emb, (size_t)emb_bytes, st);
     if (e != cudaSuccess) return set_msg(ctx, "upload failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
-    s = compute_impl(ctx, dev, out, workspace, workspace_bytes, 0, G, true, stream);
+    s = compute_impl(ctx, dev, out, workspace, workspace_bytes, 0, G, StatusInit::kClear, stream);
     if (s != GPO_OK) return s;
     if (T > 0 && (e = cudaMemcpyAsync(host_adv, out->adv, 4 * T, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
       return set_msg(ctx, "download failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
@@ -593,7 +634,7 @@ gpo_status gpo_compute_host(gpo_ctx* ctx, const gpo_batch* host, const gpo_batch
   nvtxRangePushA("gpo_compute_host pipeline");
   const bool timing = ctx->timing;  // per-stage events would interleave across the streams
   ctx->timing = false;
-  s = compute_impl(ctx, dev, out, workspace, workspace_bytes, 0, 0, true, stream);  // clears the status words
+  s = compute_impl(ctx, dev, out, workspace, workspace_bytes, 0, 0, StatusInit::kClear, stream);  // clears the status words
   cudaEvent_t* ev = ctx->pipe_ev;
   const cudaEvent_t ready = ev[2 * kPipeMaxChunks], done = ev[2 * kPipeMaxChunks + 1];
   if (s == GPO_OK) {
@@ -618,7 +659,7 @@ gpo_status gpo_compute_host(gpo_ctx* ctx, const gpo_batch* host, const gpo_batch
       if (e == cudaSuccess) e = cudaEventRecord(ev[2 * nb], ctx->pipe_in);
       const cudaStream_t cs = ctx->pipe_comp[nb % kPipeComputeStreams];
       if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ev[2 * nb], 0);
-      if (e == cudaSuccess) s = compute_impl(ctx, dev, out, workspace, workspace_bytes, ga, gb, false, cs);
+      if (e == cudaSuccess) s = compute_impl(ctx, dev, out, workspace, workspace_bytes, ga, gb, StatusInit::kKeep, cs);
       if (e == cudaSuccess && s == GPO_OK) e = cudaEventRecord(ev[2 * nb + 1], cs);
       bounds[++nb] = gb;
       ga = gb;
@@ -750,6 +791,7 @@ gpo_status gpo_loss_plan(gpo_ctx* ctx, const gpo_batch* batch, void* plan, size_
   if (e == cudaSuccess) e = launch_loss_plan(lc, *batch, loss_sizes(*batch), lp);
   ctx->nstages = 0;
   ctx->last_status = lp.status;
+  ctx->last_tag = kClearedTag;
   if (e != cudaSuccess) return set_msg(ctx, "launch failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
   return GPO_OK;
 }
@@ -816,6 +858,7 @@ gpo_status gpo_token_loss(gpo_ctx* ctx, const gpo_batch* batch, void* plan, cons
   }
   ctx->nstages = ns;
   ctx->last_status = lp.status;
+  ctx->last_tag = kClearedTag;
   if (e != cudaSuccess) return set_msg(ctx, "launch failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
   return GPO_OK;
 }
@@ -850,7 +893,8 @@ gpo_status gpo_sync_status(gpo_ctx* ctx, void* stream) {
   if (!ctx->last_status) return GPO_OK;
   e = cudaMemcpy(ctx->host_status, ctx->last_status, sizeof(uint32_t) * kStatusWords, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return set_msg(ctx, "status read failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
-  const uint32_t code = ctx->host_status[kStError];
+  const uint64_t word = (uint64_t)ctx->host_status[kStError + 1] << 32 | ctx->host_status[kStError];
+  const uint32_t code = word >> 16 == ctx->last_tag ? (uint32_t)(word & 0xFFFFu) : 0u;
   if (code != 0)
     set_msg(ctx, "%s (kernel %u, index %u)", gpo_status_string((gpo_status)code), ctx->host_status[kStWhere],
             ctx->host_status[kStDetail]);

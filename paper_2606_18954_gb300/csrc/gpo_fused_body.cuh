@@ -204,7 +204,7 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
 template <class Par>
 __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
                                                 int g, int s0, int n, bool need, Par par, int gt, int wg, int lane,
-                                                uint32_t* st) {
+                                                const Status& st) {
   int* mark = reinterpret_cast<int*>(gs->eadv);  // zeroed with the set-up
   const int pl = need ? par(gt) : -1;
   if (pl >= 0) mark[pl] = 1;
@@ -277,7 +277,7 @@ __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes&
 // butterfly.
 constexpr int kEarlyD = 1024;
 __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
-                                                int g, int s0, int n, bool tree, bool early, int lane, uint32_t* st) {
+                                                int g, int s0, int n, bool tree, bool early, int lane, const Status& st) {
   const int r = lane >> 2, c = lane & 3;
   const int nch = sz.d / 8;          // whole 16-byte chunks of a row
   const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
@@ -375,7 +375,7 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
 // every edge.  One state per group thread (kGThreads >= kMaxN); every group thread calls
 // it.  An invalid group gets bit 0 of gs->flags (visible to all on return).
 __device__ __forceinline__ void tree_setup(const gpo_batch& b, const Sizes& sz, GroupSmem* gs, int g, int r0, int nr,
-                                           int s0, int n, int gt, int wg, int lane, uint32_t* st) {
+                                           int s0, int n, int gt, int wg, int lane, const Status& st) {
   const int64_t t0 = b.group_token_off[g], t1 = b.group_token_off[g + 1];
   const int i = gt;
   int pp = -1;
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
   Ctl* ctl = reinterpret_cast<Ctl*>(smem_raw + kCtlOff);
   const uint32_t sbase = smem_u32(smem_raw);
   unsigned char* tiles = smem_raw + (((sbase + kTilesOff + 1023u) & ~1023u) - sbase);
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int KT = (sz.d + kTileK - 1) / kTileK;
   const float kappa = p.kappa_f;

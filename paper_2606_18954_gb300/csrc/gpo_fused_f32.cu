@@ -73,7 +73,7 @@ __device__ __forceinline__ bool any_block(bool f) { return __syncthreads_or(f ? 
 // that publishes the forest.
 template <int TA, int NT>
 __device__ __forceinline__ void f32_gram_links(F32Smem* gs, const float* Zs, int n, int d, int ds, int s0,
-                                               float kappa, int rule, int tid, float* part, uint32_t* st) {
+                                               float kappa, int rule, int tid, float* part, const Status& st) {
   constexpr int KS = NT / 256;  // parts of the block, each a range of k
   const int t = tid & 255, kq = tid >> 8;
   const int ti = t >> 4, tj = t & 15;
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(NT, 1) fused_f32_kernel(gpo_batch b, gpo_outpu
   extern __shared__ __align__(16) unsigned char smem_raw[];
   F32Smem* gs = reinterpret_cast<F32Smem*>(smem_raw);
   float* Zs = reinterpret_cast<float*>(smem_raw + kF32ZOff);
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int nt = NT;
   const int d = sz.d, ds = f32_row_stride(d);

@@ -25,7 +25,7 @@ __host__ __device__ inline size_t group_smem(int n) {
 template <int kPer>
 __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o, Sizes sz, Ws ws, Params p) {
   extern __shared__ __align__(16) unsigned char sm[];
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   if (aborted(st)) return;
   const int g = blockIdx.x;
   const GroupInfo gi = ws.groups[g];

@@ -27,8 +27,8 @@ constexpr int64_t kPipeMinChunkBytes = (int64_t)8 << 20;
 
 // status words (uint32) at the head of the workspace
 enum : int {
-  kStError = 0,     // first gpo_status reported by any kernel
-  kStAbort = 1,     // nonzero: kernels stop early
+  kStError = 0,     // (words 0 and 1, one 64-bit value) the call's tag << 16 | first gpo_status reported
+                    // by any kernel of the call; another tag: none
   kStItems = 2,     // number of similarity work items planned
   kStTicket = 3,    // last-block ticket of the prep kernel
   kStDetail = 4,    // first failing index (debug aid)
@@ -51,6 +51,7 @@ struct GroupInfo {
 // Device pointers into the caller's workspace (computed on the host).
 struct Ws {
   uint32_t* status;      // [kStatusWords]
+  uint64_t tag;          // the call's tag in the status words (see Status)
   Item* items;           // [max_items]: per group, its diagonal items, then its off-diagonal ones
   int* blk_ready;        // [max_items]: at a diagonal item's position, set once it has written its norms
   GroupInfo* groups;     // [G]
@@ -103,12 +104,28 @@ struct Params {
 
 // ------------------------------------------------------------------ errors
 
-__device__ __forceinline__ void report(uint32_t* st, int code, int where, int detail) {
-  if (atomicCAS(&st[kStError], 0u, (uint32_t)code) == 0u) {
-    st[kStWhere] = (uint32_t)where;
-    st[kStDetail] = (uint32_t)detail;
+// The status words of a call.  An error carries the call's 48-bit tag, so that words left by
+// earlier calls, or never written, are no error of this one: a call with a tag of its own
+// (fresh_tag on the host) needs no clearing of the words first, which as a memset node before
+// the kernel cost every call about 2 us.  Calls whose words are cleared share kClearedTag.
+struct Status {
+  uint32_t* p;
+  uint64_t tag;
+};
+constexpr uint64_t kClearedTag = 1;
+
+__device__ __forceinline__ bool aborted(const Status& st) {
+  return *reinterpret_cast<volatile const uint64_t*>(st.p + kStError) >> 16 == st.tag;
+}
+
+__device__ __forceinline__ void report(const Status& st, int code, int where, int detail) {
+  unsigned long long* w = reinterpret_cast<unsigned long long*>(st.p + kStError);
+  const unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(w);
+  if (old >> 16 == st.tag) return;  // not the call's first error
+  if (atomicCAS(w, old, (unsigned long long)st.tag << 16 | (unsigned)code) == old) {
+    st.p[kStWhere] = (uint32_t)where;
+    st.p[kStDetail] = (uint32_t)detail;
   }
-  atomicExch(&st[kStAbort], 1u);
 }
 
 // Bounds checks of the debug build (-DGPO_DEBUG, a stand-in for a device memory checker):
@@ -116,13 +133,9 @@ __device__ __forceinline__ void report(uint32_t* st, int code, int where, int de
 // with the index and the check's number (kWhere*), and the caller skips the access.  In the
 // release build it is the constant true and costs nothing.
 #ifdef GPO_DEBUG
-__device__ __forceinline__ bool bounds_ok(uint32_t* st, int64_t i, int64_t n, int where) {
+__device__ __forceinline__ bool bounds_ok(const Status& st, int64_t i, int64_t n, int where) {
   if (i >= 0 && i < n) return true;
-  if (atomicCAS(&st[kStError], 0u, (uint32_t)GPO_ERR_BOUNDS) == 0u) {
-    st[kStWhere] = (uint32_t)where;
-    st[kStDetail] = (uint32_t)i;
-  }
-  atomicExch(&st[kStAbort], 1u);
+  report(st, GPO_ERR_BOUNDS, where, (int)i);
   return false;
 }
 #define GPO_BOUNDS(st, i, n, where) ::gpo::bounds_ok((st), (int64_t)(i), (int64_t)(n), (where))
@@ -138,10 +151,6 @@ enum : int {
   kWhereNorms = 104,       // an fp32 norm of the similarity stage
   kWhereSmemRow = 105,     // a row of the fp32 group-resident kernel's shared-memory copy
 };
-
-__device__ __forceinline__ bool aborted(const uint32_t* st) {
-  return *((volatile const uint32_t*)&st[kStAbort]) != 0u;
-}
 
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
@@ -190,7 +199,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // down cleanly instead of hanging the GPU.
 // Wind-down waits (copies or MMAs still in flight before the CTA exits) pass
 // honor_abort = false so that they only stop at their time limit.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t* st, int where,
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const Status& st, int where,
                                           uint64_t limit_ns = 2000000000ull, bool honor_abort = true) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer_ns();
@@ -225,7 +234,7 @@ __device__ __forceinline__ void st_release_gpu(int* p, int v) {
 
 // Waits until *flag != 0 (acquire).  Gives up after `limit_ns` or when the abort flag
 // is raised, reporting GPO_ERR_TIMEOUT on a timeout; returns whether the flag was seen.
-__device__ __forceinline__ bool wait_flag(const int* flag, uint32_t* st, int where,
+__device__ __forceinline__ bool wait_flag(const int* flag, const Status& st, int where,
                                           uint64_t limit_ns = 2000000000ull) {
   if (ld_acquire_gpu(flag)) return true;
   const uint64_t t0 = globaltimer_ns();

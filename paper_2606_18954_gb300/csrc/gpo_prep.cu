@@ -54,7 +54,7 @@ __device__ int block_incl_scan(int x, int* warp_tot) {
 // (rollout, depth) and per-rollout group; the last block to finish plans the
 // similarity work items.  Nothing is dereferenced before its range is checked.
 __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes sz, Ws ws) {
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
   const int32_t* go = b.group_rollout_off;
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
   __shared__ int s_incl[kPlanThreads], s_s0[kPlanThreads], s_n[kPlanThreads];
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&st[kStTicket], 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) s_last = atomicAdd(&st.p[kStTicket], 1u) == gridDim.x - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
   if (threadIdx.x == 0) {
     const int total = s_carry;
     if (total > ws.max_items) report(st, GPO_ERR_WORKSPACE, 0, total);
-    st[kStItems] = aborted(st) ? 0u : (uint32_t)total;
+    st.p[kStItems] = aborted(st) ? 0u : (uint32_t)total;
   }
 }
 
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_prep_kernel(gpo_batch b, Si
   extern __shared__ int tsm[];
   __shared__ int s_wa[32];
   __shared__ long long s_wb[32];
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   const int g = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const int r0 = b.group_rollout_off[g], r1 = b.group_rollout_off[g + 1];
   const int s0 = b.group_state_off[g], s1 = b.group_state_off[g + 1];
@@ -388,7 +388,7 @@ __device__ __forceinline__ float load1(const void* base, int64_t elem) {
 
 template <bool kBf16, bool kVec>
 __global__ void __launch_bounds__(256) row_stats_kernel(gpo_batch b, Sizes sz, Ws ws) {
-  if (aborted(ws.status)) return;
+  if (aborted(Status{ws.status, ws.tag})) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(256) row_stats_kernel(gpo_batch b, Sizes sz, W
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     if (lane == 0) {
-      if (!isfinite(s2)) report(ws.status, GPO_ERR_NONFINITE, 1, (int)row);
+      if (!isfinite(s2)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 1, (int)row);
       ws.nrm2[row] = s2;
       ws.rn[row] = s2 > 0.f ? 1.0f / sqrtf(s2) : 0.f;
     }
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
       float2 n2, dot;
       exact_pair_sums<kBf16>(b.root_emb, g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
       if (lane == 0) {
-        if (!isfinite(n2.x)) report(ws.status, GPO_ERR_NONFINITE, 3, (int)job);
+        if (!isfinite(n2.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, (int)job);
         ws.x_root_n2[g] = n2;
       }
       continue;
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
     float2 n2, dot;
     exact_pair_sums<kBf16>(b.emb, (int64_t)v * sz.stride, pbase, poff, pbase != nullptr, sz.d, lane, n2, dot);
     if (lane == 0) {
-      if (!isfinite(n2.x) || !isfinite(dot.x)) report(ws.status, GPO_ERR_NONFINITE, 3, v);
+      if (!isfinite(n2.x) || !isfinite(dot.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, v);
       ws.x_n2[v] = n2;
       ws.x_dot[v] = dot;
       if (!kBf16) {  // the norms of the threshold test (bf16: from the similarity stage or row_stats)
@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Size
     }
     if (p == -1) dot = make_float2(0.f, 0.f);
     if (live && j == 0) {
-      if (!isfinite(n2.x) || !isfinite(dot.x)) report(ws.status, GPO_ERR_NONFINITE, 3, (int)v);
+      if (!isfinite(n2.x) || !isfinite(dot.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, (int)v);
       ws.x_n2[v] = n2;
       ws.x_dot[v] = dot;
     }
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, 
     float2 n2, dot;
     exact_pair_sums<true>(b.root_emb, g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
     if (lane == 0) {
-      if (!isfinite(n2.x)) report(ws.status, GPO_ERR_NONFINITE, 3, (int)(sz.N + g));
+      if (!isfinite(n2.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, (int)(sz.N + g));
       ws.x_root_n2[g] = n2;
     }
   }
@@ -810,7 +810,7 @@ cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Si
 // with 16-byte stores in its aligned middle and scalar stores at the ends.
 
 __global__ void __launch_bounds__(256) tokens_kernel(gpo_batch b, gpo_outputs o, Sizes sz, Ws ws) {
-  if (aborted(ws.status)) return;
+  if (aborted(Status{ws.status, ws.tag})) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(256) tokens_kernel(gpo_batch b, gpo_outputs o,
       const int64_t s = __shfl_sync(0xffffffffu, ts, j);
       const int64_t e = s + __shfl_sync(0xffffffffu, L, j);
       const float a = __shfl_sync(0xffffffffu, va, j);
-      if (!GPO_BOUNDS(ws.status, e - 1, sz.T, kWhereTokens) || !GPO_BOUNDS(ws.status, s, sz.T, kWhereTokens)) continue;
+      if (!GPO_BOUNDS((Status{ws.status, ws.tag}), e - 1, sz.T, kWhereTokens) || !GPO_BOUNDS((Status{ws.status, ws.tag}), s, sz.T, kWhereTokens)) continue;
       write_span(o.adv, s, e, a, lane);
       if (o.adv_cor) write_span(o.adv_cor, s, e, __shfl_sync(0xffffffffu, vc, j), lane);
       if (o.adv_eff) write_span(o.adv_eff, s, e, __shfl_sync(0xffffffffu, ve, j), lane);

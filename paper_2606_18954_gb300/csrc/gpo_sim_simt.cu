@@ -197,9 +197,9 @@ template <bool kBf16>
 __global__ void __launch_bounds__(kThreads) sim_simt_kernel(gpo_batch b, Sizes sz, Ws ws, float kappa, int rule) {
   extern __shared__ __align__(16) unsigned char simt_smem[];
   SimtSmem& sm = *reinterpret_cast<SimtSmem*>(simt_smem);
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   const int it = blockIdx.x / kSubs, sub = blockIdx.x % kSubs;
-  const int nitems = (int)*((volatile uint32_t*)&st[kStItems]);
+  const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
   if (it >= nitems || aborted(st)) return;
   const Item item = ws.items[it];
   const GroupInfo gi = ws.groups[item.group];

@@ -116,11 +116,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t sbase = smem_u32(smem_raw);
   constexpr uint32_t kCtlBytes = (sizeof(SmemCtl) + 15) & ~15u;
   unsigned char* tiles = smem_raw + (((sbase + kCtlBytes + 1023u) & ~1023u) - sbase);
-  uint32_t* st = ws.status;
+  const Status st{ws.status, ws.tag};
   const bool tree = ws.tree_end != nullptr;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nitems = (int)*((volatile uint32_t*)&st[kStItems]);
+  const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
   if (aborted(st) || nitems == 0 || (int)blockIdx.x >= nitems) return;
   const int KT = (sz.d + kTileK - 1) / kTileK;
 
