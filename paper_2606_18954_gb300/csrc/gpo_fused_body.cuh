@@ -18,6 +18,7 @@ constexpr int kEdgeList = kWarpEdges * (kEpiThreads / 32);
 constexpr int kBarGroup = 1;                    // named barrier of the group warps
 constexpr int kBarEpi = 2;                      // named barrier of the drain warps
 constexpr int kBarSetup = 3;                    // named barrier of warps 2 and 3 (early set-up)
+static_assert(kMaxN <= 3 * kTileM, "row blocks of a group");
 static_assert(kThreads % 128 == 0 && kThreads >= 256 && kGThreads >= kMaxN, "fused kernel shape");
 
 struct Seg {
@@ -44,42 +45,40 @@ __device__ __forceinline__ int r32(int x) { return (x + 31) & ~31; }
 // fit 512 TMEM columns, else pass 0 = blocks >= 1 (at most 256 + 128 columns)
 // and pass 1 = block 0 (at most 256 + 128), so that the norms of every column
 // a pass needs come from its own or an earlier pass.
-__device__ __forceinline__ void make_plan(int n, Plan& pl) {
-  Seg all[4];
-  int na = 0, tot = 0;
+// The roles that run in single lanes (producer, MMA issuer) and the drain's plan in shared memory
+// take all of this without local arrays: those would lie in local memory, for which the
+// statistics' streaming loads leave no place in the few KB of L1 beside the tile ring, so that
+// every k-slice of those roles waited for L2 (128 groups of 256 states 55.2 -> 52.3 us, 512 of
+// 320 252 -> 243).
+
+// Passes of a group with n states.
+__device__ __forceinline__ int plan_passes(int n) {
+  int tot = 0;
   for (int b = 0; b * kTileM < n; ++b)
-    for (int c0 = b * kTileM; c0 < n && na < 4; c0 += kTileN) {
-      all[na].b = b;
-      all[na].c0 = c0;
-      all[na].len = min(kTileN, n - c0);
-      tot += r32(all[na].len);
-      ++na;
-    }
-  pl.nseg[0] = pl.nseg[1] = 0;
-  if (tot <= kTmemCols) {
-    pl.npass = 1;
-    int col = 0;
-    for (int i = 0; i < na; ++i) {
-      Seg s = all[i];
-      s.tcol = col;
-      col += r32(s.len);
-      pl.seg[0][pl.nseg[0]++] = s;
-    }
-  } else {
-    pl.npass = 2;
-    int col0 = 0, col1 = 0;
-    for (int i = 0; i < na; ++i) {
-      Seg s = all[i];
-      if (s.b >= 1) {
-        s.tcol = col0;
-        col0 += r32(s.len);
-        pl.seg[0][pl.nseg[0]++] = s;
-      } else {
-        s.tcol = col1;
-        col1 += r32(s.len);
-        pl.seg[1][pl.nseg[1]++] = s;
+    for (int c0 = b * kTileM; c0 < n; c0 += kTileN) tot += r32(min(kTileN, n - c0));
+  return tot <= kTmemCols ? 1 : 2;
+}
+// Row blocks [b0, b1) of a pass (fewer where the group ends before).
+__device__ __forceinline__ void pass_blocks(int npass, int pass, int& b0, int& b1) {
+  b0 = npass == 2 && pass == 0 ? 1 : 0;
+  b1 = npass == 2 && pass == 1 ? 1 : 3;
+}
+
+__device__ __forceinline__ void make_plan(int n, Plan& pl) {
+  pl.npass = plan_passes(n);
+  for (int pass = 0; pass < pl.npass; ++pass) {
+    int b0, b1, m = 0, col = 0;
+    pass_blocks(pl.npass, pass, b0, b1);
+    for (int b = b0; b < b1 && b * kTileM < n; ++b)
+      for (int c0 = b * kTileM; c0 < n; c0 += kTileN) {
+        Seg& sg = pl.seg[pass][m++];  // at most 4: two of block 0, one each of blocks 1 and 2
+        sg.b = b;
+        sg.c0 = c0;
+        sg.len = min(kTileN, n - c0);
+        sg.tcol = col;
+        col += r32(sg.len);
       }
-    }
+    pl.nseg[pass] = m;
   }
 }
 
@@ -152,6 +151,7 @@ struct __align__(8) Ctl {
   uint64_t tfull;
   uint64_t tempty;
   uint64_t drain;
+  int slice_off[kMaxSlots];  // the producer's: offsets of the slices in flight
   uint32_t tmem_base;
 };
 
@@ -530,7 +530,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     // Otherwise wait for the oldest slice's consumption and look again.
     int head = 0;
     uint32_t seq = 0, oldest = 0;  // slices issued; oldest slice not yet seen consumed
-    int f_off[kMaxSlots];
     bool ok = true;
     // L2 policy: pass 0 of a two-pass group keeps its rows (pass 1 reads them again),
     // pass 1 drops them first (their last read)
@@ -538,17 +537,16 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     for (int g = sz.g0 + (int)blockIdx.x; g < sz.g1 && ok; g += gridDim.x) {
       int r0, nr, s0, n;
       if (!group_active(b, sz, g, r0, nr, s0, n)) continue;
-      Plan pl;
-      make_plan(n, pl);
+      const int npass = plan_passes(n);
       const int rows = r32(n);  // rows [0, r32(n)) of the group; the MMAs read no further
-      for (int pass = 0; pass < pl.npass && ok; ++pass) {
-        const int row0 = pl.npass == 2 && pass == 0 ? kTileM : 0;  // pass 0 of two never reads block 0
+      for (int pass = 0; pass < npass && ok; ++pass) {
+        const int row0 = npass == 2 && pass == 0 ? kTileM : 0;  // pass 0 of two never reads block 0
         const int bytes = (rows - row0) * 128;
-        const int hint = pl.npass == 1 ? 0 : (pass == 0 ? 1 : 2);
+        const int hint = npass == 1 ? 0 : (pass == 0 ? 1 : 2);
         for (int k = 0; k < KT && ok; ++k) {
           const int off = ring_place(head, bytes);
           while (oldest < seq) {
-            const int o = f_off[oldest % kMaxSlots];
+            const int o = ctl->slice_off[oldest % kMaxSlots];
             const bool busy = seq - oldest >= (uint32_t)kMaxSlots ||
                               (o < head ? (off != head && off + bytes > o) : (off != head || head + bytes > o));
             if (!busy) break;
@@ -571,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
                                hint == 1 ? keep : drop);
             r += big ? kTileM : kTailRows;
           }
-          f_off[bi] = off;
+          ctl->slice_off[bi] = off;
           head = off + bytes;
           ++seq;
         }
@@ -597,11 +595,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     for (int g = sz.g0 + (int)blockIdx.x; g < sz.g1 && ok; g += gridDim.x) {
       int r0, nr, s0, n;
       if (!group_active(b, sz, g, r0, nr, s0, n)) continue;
-      Plan pl;
-      make_plan(n, pl);
+      const int npass = plan_passes(n);
       const int rows = r32(n);
-      for (int pass = 0; pass < pl.npass && ok; ++pass, ++u) {
-        const int row0 = pl.npass == 2 && pass == 0 ? kTileM : 0;
+      for (int pass = 0; pass < npass && ok; ++pass, ++u) {
+        const int row0 = npass == 2 && pass == 0 ? kTileM : 0;
+        int b0, b1;  // the pass's segments as make_plan has them, walked
+        pass_blocks(npass, pass, b0, b1);
         const int bytes = (rows - row0) * 128;
         if (!mbar_wait(&ctl->tempty, ((uint32_t)u & 1u) ^ 1u, st, 22)) {
           ok = false;
@@ -618,14 +617,18 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           }
           tc_fence_after();
           const uint32_t t = smem_u32(tiles + off);
-          for (int si = 0; si < pl.nseg[pass]; ++si) {
-            const Seg sg = pl.seg[pass][si];
-            const uint64_t ad = smem_desc_k128(t + (uint32_t)((sg.b * kTileM - row0) * 128));
-            const uint64_t bd = smem_desc_k128(t + (uint32_t)((sg.c0 - row0) * 128));
-            const uint32_t idesc = idesc_bf16_f32(kTileM, r16(sg.len));
+          uint32_t dt = tmem;
+          for (int b = b0; b < b1 && b * kTileM < n; ++b) {
+            const uint64_t ad = smem_desc_k128(t + (uint32_t)((b * kTileM - row0) * 128));
+            for (int c0 = b * kTileM; c0 < n; c0 += kTileN) {
+              const int len = min(kTileN, n - c0);
+              const uint64_t bd = smem_desc_k128(t + (uint32_t)((c0 - row0) * 128));
+              const uint32_t idesc = idesc_bf16_f32(kTileM, r16(len));
 #pragma unroll
-            for (int kk = 0; kk < kTileK / 16; ++kk)
-              mma_bf16_ss(tmem + (uint32_t)sg.tcol, ad + 2u * kk, bd + 2u * kk, idesc, (k | kk) != 0);
+              for (int kk = 0; kk < kTileK / 16; ++kk)
+                mma_bf16_ss(dt, ad + 2u * kk, bd + 2u * kk, idesc, (k | kk) != 0);
+              dt += (uint32_t)r32(len);
+            }
           }
           mma_commit(&ctl->empty[bi]);
           ++seq;

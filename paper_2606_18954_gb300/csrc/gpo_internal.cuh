@@ -627,24 +627,10 @@ __device__ __forceinline__ void half_warp_row_sums(const uint4* x, const uint4* 
   if ((okm & half) != half) {  // this half again, by TwoSum
     uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
 #pragma unroll 1
-    for (int k = hl; k < nch; k += 16) {
-      const uint4 a = x[k];
-      uint4 b = make_uint4(0u, 0u, 0u, 0u);
-      if (kDot) b = y[k];
-      const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll 1
-      for (int h = 0; h < 4; ++h) {
-        const uint64_t xx = bf16x2_f32x2(aw[h]);
-        f2_acc(ns, ne, f2mul(xx, xx));
-        if (kDot) f2_acc(ds, de, f2mul(xx, bf16x2_f32x2(bw[h])));
-      }
-    }
-    if (tail) {
-      for (int k = 8 * nch; k < d; ++k) {
-        const uint64_t xx = pack_f2((uint32_t)xr[k] << 16, 0u);
-        f2_acc(ns, ne, f2mul(xx, xx));
-        if (kDot) f2_acc(ds, de, f2mul(xx, pack_f2((uint32_t)yr[k] << 16, 0u)));
-      }
+    for (int k = hl; k < d; k += 16) {
+      const uint64_t xx = pack_f2((uint32_t)xr[k] << 16, 0u);
+      f2_acc(ns, ne, f2mul(xx, xx));
+      if (kDot) f2_acc(ds, de, f2mul(xx, pack_f2((uint32_t)yr[k] << 16, 0u)));
     }
     pn = f2_finish(ns, ne);
     pd = f2_finish(ds, de);

@@ -152,8 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
     int stage = 0;
     uint32_t phase = 0;
-    int last_parity[kStages];
-    for (int s = 0; s < kStages; ++s) last_parity[s] = -1;
+    uint32_t issued = 0;  // k-slices
     bool ok = true;
     for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
       const Item item = ws.items[it];
@@ -167,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         unsigned char* sa = tiles + stage * kStageBytes;
         unsigned char* sb = sa + kBoxBytes;
         mbar_arrive_expect_tx(&ctl->full[stage], (uint32_t)(nbox * kBoxBytes));
-        last_parity[stage] = (int)phase;
+        ++issued;
         const int x = k * kTileK;
         tma_load_2d(sa, &zmap, &ctl->full[stage], x, item.row0);
         if (diag) {
@@ -183,8 +182,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     // wind-down: every issued copy must land before the CTA may exit
-    for (int s = 0; s < kStages; ++s)
-      if (last_parity[s] >= 0) mbar_wait(&ctl->full[s], (uint32_t)last_parity[s], st, 11, 200000000ull, false);
+    for (uint32_t s = 0; s < kStages; ++s)  // the parity of each stage's last use
+      if (s < issued) mbar_wait(&ctl->full[s], (issued - 1 - s) / kStages & 1u, st, 11, 200000000ull, false);
     }
     __syncwarp();
   } else if (warp == 1) {
