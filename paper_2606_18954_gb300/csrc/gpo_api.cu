@@ -478,17 +478,20 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
     if (e == cudaSuccess) e = stage("prep", [&] { return launch_prep(lc, b, sz, ws); });
     if (e == cudaSuccess && sz.N > 0) {
       // the fp32 norms of the threshold test come from the Gram tiles (tcgen05), from the
-      // compensated statistics (fp32 embeddings, first then) or from row_stats; bf16 embeddings'
-      // statistics follow the similarity stage or row_stats, whose norms give their sums' biases
+      // compensated statistics (fp32 embeddings, first then) or from row_stats; the tensor-core
+      // kernel computes the compensated statistics beside the similarities, bf16 embeddings on
+      // the CUDA cores take theirs after row_stats, whose norms give the sums' biases
       const bool exact_first = !use_tc && !bud && b.emb_dtype == GPO_EMB_F32;
       auto exact = [&] { return launch_exact_stats(lc, b, sz, ws, true); };
-      if (exact_first) e = stage("exact_stats", exact);
-      else if (!use_tc) e = stage("row_stats", [&] { return launch_row_stats(lc, b, sz, ws); });
-      if (e == cudaSuccess)
-        e = stage("similarity", [&] {
-          return use_tc ? launch_sim_tc(lc, map, b, sz, ws, pp) : launch_sim_simt(lc, b, sz, ws, pp);
-        });
-      if (e == cudaSuccess && !bud && !exact_first) e = stage("exact_stats", exact);
+      if (use_tc) {
+        if (b.root_emb && !bud) e = stage("root_norms", [&] { return launch_root_norms(lc, b, sz, ws); });
+        if (e == cudaSuccess) e = stage("similarity", [&] { return launch_sim_tc(lc, map, b, sz, ws, pp, !bud); });
+      } else {
+        if (exact_first) e = stage("exact_stats", exact);
+        else e = stage("row_stats", [&] { return launch_row_stats(lc, b, sz, ws); });
+        if (e == cudaSuccess) e = stage("similarity", [&] { return launch_sim_simt(lc, b, sz, ws, pp); });
+        if (e == cudaSuccess && !bud && !exact_first) e = stage("exact_stats", exact);
+      }
       if (e == cudaSuccess) e = stage("groups", [&] { return launch_groups(lc, b, *out, sz, ws, pp); });
       if (e == cudaSuccess && !bud) e = stage("tokens", [&] { return launch_tokens(lc, b, *out, sz, ws); });
     }

@@ -267,19 +267,14 @@ __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes&
 // 60.1, 1024 60.0 / 58.0, 2048 111 / 95; 256 groups of 56: d = 256 27.2 / 33.4, 768 34.4 / 37.5,
 // 1024 39.5 / 39.6, 2048 58.0 / 51.9).  A branching batch reads 0.85 of its eta's (tree, d =
 // 1024: 71.0 / 74.4).  The calling warps claim blocks of 8 rows from gs->nstat[0] until none is
-// left, so that warps that join late or run slower take fewer; lane 4 r + c takes every fourth
-// 16-byte chunk of row r from chunk c; a parent that is the row before comes from the lane 4
-// below, other parents and the prompt embedding are loaded.  Parents: with `early` (chain
+// left, so that warps that join late or run slower take fewer (eight_rows_sums).  Parents: with `early` (chain
 // layout, before the group's set-up) the previous state for every state but the group's first
 // (the set-up fixes the rollouts' first states afterwards: their parent is the prompt root);
-// otherwise from the group layout in shared memory.  bf16 products are exact in fp32, sums by
-// TwoSum (no bound of the norms is known yet), the row's 4 partial pairs combined in a fixed
-// butterfly.
+// otherwise from the group layout in shared memory.
 constexpr int kEarlyD = 1024;
 __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
                                                 int g, int s0, int n, bool tree, bool early, int lane, const Status& st) {
   const int r = lane >> 2, c = lane & 3;
-  const int nch = sz.d / 8;          // whole 16-byte chunks of a row
   const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
   const uint4* Z = reinterpret_cast<const uint4*>(b.emb);
   const uint4* RZ = reinterpret_cast<const uint4*>(b.root_emb);
@@ -309,57 +304,8 @@ __device__ __forceinline__ void group_row_stats(const gpo_batch& b, const Sizes&
     if (!__all_sync(0xffffffffu, rows_ok)) continue;
     const uint4* zb = Z + (int64_t)(s0 + (live ? i : 0)) * rs;
     const uint4* pb = pl >= 0 ? Z + (int64_t)(s0 + pl) * rs : (pl == -2 ? RZ + (int64_t)g * rs : nullptr);
-    uint64_t ns = 0ull, ne = 0ull, ds = 0ull, de = 0ull;
-    // two stages of kU chunks per lane, software-pipelined: the next stage's loads are in
-    // flight while this one's sums run (no register copies between the stages)
-    constexpr int kU = 2;
-    auto load = [&](int k0, uint4 (&x)[kU], uint4 (&y)[kU]) {
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int k = k0 + 4 * u + c;
-        const bool in = k < nch;
-        x[u] = live && in ? zb[k] : make_uint4(0u, 0u, 0u, 0u);
-        y[u] = !from_left && pb && in ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
-      }
-    };
-    auto accumulate = [&](uint4 (&x)[kU], uint4 (&y)[kU]) {
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        uint4 t;
-        t.x = __shfl_up_sync(0xffffffffu, x[u].x, 4);
-        t.y = __shfl_up_sync(0xffffffffu, x[u].y, 4);
-        t.z = __shfl_up_sync(0xffffffffu, x[u].z, 4);
-        t.w = __shfl_up_sync(0xffffffffu, x[u].w, 4);
-        if (from_left) y[u] = t;
-        const uint32_t xw[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yw[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const uint64_t xx = bf16x2_f32x2(xw[h]), yy = bf16x2_f32x2(yw[h]);
-          f2_acc(ns, ne, f2mul(xx, xx));  // bf16 products are exact in fp32
-          f2_acc(ds, de, f2mul(xx, yy));
-        }
-      }
-    };
-    uint4 xa[kU], ya[kU], xb[kU], yb[kU];
-    load(0, xa, ya);
-#pragma unroll 1
-    for (int k0 = 0; k0 < nch; k0 += 8 * kU) {
-      load(k0 + 4 * kU, xb, yb);  // past the row's end: zeros, which add nothing
-      accumulate(xa, ya);
-      load(k0 + 8 * kU, xa, ya);
-      accumulate(xb, yb);
-    }
-    if (sz.d % 8 != 0 && c == 0 && live) {  // the ragged end of the row, one lane per row
-      const uint16_t* zr = reinterpret_cast<const uint16_t*>(zb);
-      const uint16_t* pr = reinterpret_cast<const uint16_t*>(pb);
-      for (int k = 8 * nch; k < sz.d; ++k) {
-        const uint64_t xx = pack_f2((uint32_t)zr[k] << 16, 0u);  // one fp32 lane (the other stays 0)
-        f2_acc(ns, ne, f2mul(xx, xx));
-        f2_acc(ds, de, f2mul(xx, pack_f2(pr ? (uint32_t)pr[k] << 16 : 0u, 0u)));
-      }
-    }
-    const float2 n2 = lanes_pair_sum<4>(f2_finish(ns, ne));
-    float2 dot = lanes_pair_sum<4>(f2_finish(ds, de));
+    float2 n2, dot;
+    eight_rows_sums<false>(zb, pb, live, from_left, sz.d, c, 0.f, 0.f, n2, dot);
     if (pl == -1) dot = make_float2(0.f, 0.f);
     if (live && c == 0 && GPO_BOUNDS(st, s0 + i, sz.N, kWhereStats)) {
       ws.x_n2[s0 + i] = n2;

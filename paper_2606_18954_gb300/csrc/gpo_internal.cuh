@@ -639,6 +639,88 @@ __device__ __forceinline__ void half_warp_row_sums(const uint4* x, const uint4* 
   dot = kDot ? lanes_pair_sum<16>(pd) : pd;
 }
 
+// |x|^2 and <x, y> as float pairs of eight bf16 rows of d elements (16-byte aligned) by one warp,
+// the row at zb with its parent's at pb (null: none, the dot is then 0): lane 4 r + c takes
+// every fourth 16-byte chunk of row r from chunk c, two stages of kU chunks software-pipelined.
+// from_left: the parent is the row of the lanes 4 below, whose chunks come by shuffle.  bf16
+// products are exact in fp32; the row's 4 partial pairs are combined in a fixed butterfly.
+//   kNorms = false: sums by TwoSum (no bound of the norms is known).
+//   kNorms = true: biased sums, with the biases from the fp32 squared norms nx, ny of the rows, good
+//   to far better than 1 %; if a sum leaves its bias's range (a norm that was not what it was
+//   taken for), the warp's rows again by TwoSum, for those rows.
+template <bool kNorms>
+__device__ __forceinline__ void eight_rows_sums(const uint4* zb, const uint4* pb, bool live, bool from_left, int d,
+                                                int c, float nx, float ny, float2& n2, float2& dot) {
+  const int nch = d / 8;  // whole 16-byte chunks of a row
+  BiasedSum sn, sd;       // (TwoSum: only s0 and e0, from zero)
+  bs_init(sn, kNorms ? pow2_ceil(4.04f * nx) : 0.f);
+  bs_init(sd, kNorms ? pow2_ceil(4.04f * (sqrtf(nx) * sqrtf(ny))) : 0.f);
+  auto add = [](BiasedSum& a, uint64_t x, uint64_t y, bool odd) {
+    if (!kNorms) f2_acc(a.s0, a.e0, f2mul(x, y));
+    else if (odd) biased_add(a.s1, a.e1, x, y);
+    else biased_add(a.s0, a.e0, x, y);
+  };
+  constexpr int kU = 2;
+  auto load = [&](int k0, uint4 (&x)[kU], uint4 (&y)[kU]) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int k = k0 + 4 * u + c;
+      const bool in = k < nch;
+      x[u] = live && in ? zb[k] : make_uint4(0u, 0u, 0u, 0u);
+      y[u] = !from_left && pb && in ? pb[k] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  auto accumulate = [&](uint4 (&x)[kU], uint4 (&y)[kU]) {
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      uint4 t;
+      t.x = __shfl_up_sync(0xffffffffu, x[u].x, 4);
+      t.y = __shfl_up_sync(0xffffffffu, x[u].y, 4);
+      t.z = __shfl_up_sync(0xffffffffu, x[u].z, 4);
+      t.w = __shfl_up_sync(0xffffffffu, x[u].w, 4);
+      if (from_left) y[u] = t;
+      const uint32_t xw[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, yw[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const uint64_t xx = bf16x2_f32x2(xw[h]), yy = bf16x2_f32x2(yw[h]);
+        add(sn, xx, xx, h & 1);
+        add(sd, xx, yy, h & 1);
+      }
+    }
+  };
+  uint4 xa[kU], ya[kU], xb[kU], yb[kU];
+  load(0, xa, ya);
+#pragma unroll 1
+  for (int k0 = 0; k0 < nch; k0 += 8 * kU) {
+    load(k0 + 4 * kU, xb, yb);  // past the row's end: zeros, which add nothing
+    accumulate(xa, ya);
+    load(k0 + 8 * kU, xa, ya);
+    accumulate(xb, yb);
+  }
+  if (d % 8 != 0 && c == 0 && live) {  // the ragged end of the row, one lane per row
+    const uint16_t* zr = reinterpret_cast<const uint16_t*>(zb);
+    const uint16_t* pr = reinterpret_cast<const uint16_t*>(pb);
+    for (int k = 8 * nch; k < d; ++k) {
+      const uint64_t xx = pack_f2((uint32_t)zr[k] << 16, 0u);  // one fp32 lane (the other stays 0)
+      add(sn, xx, xx, false);
+      add(sd, xx, pack_f2(pr ? (uint32_t)pr[k] << 16 : 0u, 0u), false);
+    }
+  }
+  n2 = lanes_pair_sum<4>(kNorms ? bs_pair(sn) : f2_finish(sn.s0, sn.e0));
+  dot = lanes_pair_sum<4>(kNorms ? bs_pair(sd) : f2_finish(sd.s0, sd.e0));
+  if constexpr (kNorms) {
+    const uint32_t okm = __ballot_sync(0xffffffffu, !live || (bs_in_range(sn) && bs_in_range(sd)));
+    if (okm != 0xffffffffu) {  // (warp-uniform)
+      float2 n2t, dott;
+      eight_rows_sums<false>(zb, pb, live, from_left, d, c, 0.f, 0.f, n2t, dott);
+      if (((okm >> (threadIdx.x & 28)) & 15u) != 15u) {
+        n2 = n2t;
+        dot = dott;
+      }
+    }
+  }
+}
+
 // One warp: |z|^2 of the row at element offset zrow of `base` and, if has_p, its dot with
 // the row at poff of `pbase`, as float pairs.  bf16 products are exact in fp32, fp32
 // products are split by TwoProduct, sums are compensated (Sum2) per lane and the lanes'
@@ -755,11 +837,14 @@ cudaError_t launch_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz
 // with_norms: ws.nrm2 holds every row's fp32 squared norm (the similarity stage ran first)
 cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                                bool with_norms = false);
+// |prompt embedding|^2 of groups [g0, g1) into ws.x_root_n2 (bf16)
+cudaError_t launch_root_norms(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
 cudaError_t launch_tree_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
 cudaError_t setup_tree_prep();
 cudaError_t launch_row_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
+// stats: the kernel computes every row's compensated statistics too
 cudaError_t launch_sim_tc(const LaunchCtx& lc, const CUtensorMap& map, const gpo_batch& b, const Sizes& sz,
-                          const Ws& ws, const Params& p);
+                          const Ws& ws, const Params& p, bool stats);
 cudaError_t launch_sim_simt(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                             const Params& p);
 cudaError_t launch_groups(const LaunchCtx& lc, const gpo_batch& b, const gpo_outputs& o, const Sizes& sz,

@@ -772,6 +772,14 @@ __global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, 
   }
 }
 
+cudaError_t launch_root_norms(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws) {
+  int64_t blocks = ((int64_t)(sz.g1 - sz.g0) + 7) / 8;
+  if (blocks < 1) return cudaSuccess;
+  if (blocks > (int64_t)lc.num_sms * 8) blocks = (int64_t)lc.num_sms * 8;
+  root_norms_kernel<<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                                bool with_norms) {
   const int64_t jobs = (int64_t)sz.N + (b.root_emb ? sz.G : 0);  // at most (range calls take fewer)
@@ -782,10 +790,9 @@ cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Si
     int64_t blocks = ((int64_t)sz.N + 63) / 64;  // a warp per 8 rows
     const int64_t bcap = (int64_t)lc.num_sms * 32;
     blocks = blocks < 1 ? 1 : (blocks > bcap ? bcap : blocks);
-    if (b.root_emb && sz.g1 > sz.g0) {  // first: the norms-based path reads them
-      int64_t rblocks = ((int64_t)(sz.g1 - sz.g0) + 7) / 8;
-      if (rblocks > (int64_t)lc.num_sms * 8) rblocks = (int64_t)lc.num_sms * 8;
-      root_norms_kernel<<<(int)rblocks, 256, 0, lc.stream>>>(b, sz, ws);
+    if (b.root_emb) {  // first: the norms-based path reads them
+      const cudaError_t e = launch_root_norms(lc, b, sz, ws);
+      if (e != cudaSuccess) return e;
     }
     if (with_norms)
       exact_stats_lane_kernel<true><<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws);

@@ -27,6 +27,13 @@
 //                      hook-and-shortcut rounds in shared memory, and the item's
 //                      spanning forest (<= 383 edges, state -> smallest state of
 //                      its class) written out.
+//   warps 2, 3, 16..19  the compensated row statistics (|z_v|^2 and <z_{p(v)}, z_v> of every
+//                      state, 8 rows per warp at a time, eight_rows_sums), read from L2 or HBM
+//                      beside the tensor cores' work, whose pace does not depend on them, once
+//                      the rows' blocks have their norms (the biases of the sums).  64 groups of
+//                      2048 states, d = 2048: 405 us with them and 356 without, against a launch of their own of
+//                      157 us after it (two such warps 840 us, ten 414; TwoSum, which needs no
+//                      norms, 451)
 // The Gram block Z_g Z_g^T is never written to memory.
 #include "gpo_internal.cuh"
 
@@ -35,7 +42,7 @@ namespace gpo {
 namespace {
 
 constexpr int kStages = 4;
-constexpr int kThreads = 512;
+constexpr int kThreads = 640;
 constexpr int kBoxBytes = kTileM * 128;            // one 128-row x 128-byte box
 constexpr int kStageBytes = 3 * kBoxBytes;         // A box + two B boxes
 constexpr int kSlots = kTileM + kTileN;            // local union-find slots
@@ -43,6 +50,7 @@ constexpr int kTmemCols = 512;                     // two accumulators of 256 co
 constexpr int kEpiBarrier = 1;                     // named barrier of the epilogue warps
 constexpr int kEpiThreads = 384;                   // warps 4..15
 constexpr int kEpiWarps = kEpiThreads / 32;
+constexpr int kStatWarps = 6;                      // warps 2, 3 and 16..19
 constexpr int kWarpEdges = 256;                    // linked pairs listed per epilogue warp and item
 
 struct __align__(8) SmemCtl {
@@ -106,9 +114,20 @@ __device__ __forceinline__ void lunion(int* p, int a, int b) {
   }
 }
 
+// The group of rollout r: the last g < n with off[g] <= r.
+__device__ __forceinline__ int group_of_rollout(const int32_t* off, int n, int r) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off[mid] <= r) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
-    sim_tc_kernel(const __grid_constant__ CUtensorMap zmap, const int32_t* __restrict__ rollout_step_off, Sizes sz,
-                  Ws ws, float kappa, int rule, int debug_timeout) {
+    sim_tc_kernel(const __grid_constant__ CUtensorMap zmap, gpo_batch b, Sizes sz, Ws ws, float kappa, int rule,
+                  int stats, int debug_timeout) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // control block first, then the tiles on a 1024-byte boundary (128B swizzle); both are
   // smem_raw plus an offset, so the compiler keeps the shared address space
@@ -121,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
-  if (aborted(st) || nitems == 0 || (int)blockIdx.x >= nitems) return;
+  if (aborted(st) || nitems == 0) return;  // (a CTA without items has its share of the statistics)
   const int KT = (sz.d + kTileK - 1) / kTileK;
 
   if (threadIdx.x == 0) {
@@ -233,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_wait(&ctl->drain, 0, st, 14, 200000000ull, false);
     }
     __syncwarp();
-  } else if (warp >= 4) {
+  } else if (warp >= 4 && warp < 4 + kEpiWarps) {
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3;            // TMEM lane quarter
     const int rep = (warp - 4) >> 2;   // 0..2: which of the quarter's three warps
@@ -264,7 +283,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int re = send, di = -1;
       if (row < send) {
         const int2 mt = ws.state_meta[row];
-        re = tree ? ws.tree_end[row] : rollout_step_off[mt.x + 1];
+        re = tree ? ws.tree_end[row] : b.rollout_step_off[mt.x + 1];
         di = mt.y;
       }
       float thr = __int_as_float(0x7f800000);  // kappa |z_i|; +inf for a zero or absent row
@@ -432,6 +451,47 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
 
+  else if (stats) {
+    // ------------------------------------------------------------ compensated row statistics
+    const int sw = warp < 4 ? warp - 2 : warp - 4 - kEpiWarps + 2;  // 0..kStatWarps - 1
+    const int r = lane >> 2, c = lane & 3;
+    const int64_t rs = sz.stride / 8;  // row stride in 16-byte chunks
+    const uint4* Z = reinterpret_cast<const uint4*>(b.emb);
+    const uint4* RZ = reinterpret_cast<const uint4*>(b.root_emb);
+    const int nblk = (sz.N + 7) / 8;
+    for (int blk = sw * (int)gridDim.x + (int)blockIdx.x; blk < nblk; blk += kStatWarps * (int)gridDim.x) {
+      const int64_t v = (int64_t)blk * 8 + r;
+      const bool live = v < sz.N;
+      int64_t pv = -1;  // the parent's row, -1: the prompt root
+      int g = -1;       // the row's group
+      float nx = 0.f, ny = 0.f;
+      bool ready = true;
+      if (live) {
+        const int2 mt = ws.state_meta[v];
+        if (tree) pv = ws.tree_par[v];
+        else if (mt.y > 1) pv = v - 1;
+        g = tree ? mt.x : group_of_rollout(b.group_rollout_off, sz.G, mt.x);
+        // the rows' norms (biases of the sums) come from their blocks' diagonal items
+        const GroupInfo gi = ws.groups[g];
+        const int bv = (int)(v - gi.s0) / kTileM, bp = pv >= 0 ? (int)(pv - gi.s0) / kTileM : bv;
+        ready = wait_flag(ws.blk_ready + gi.blk0 + bv, st, 18) && wait_flag(ws.blk_ready + gi.blk0 + bp, st, 18);
+        if (ready) {
+          nx = __ldcg(ws.nrm2 + v);
+          ny = pv >= 0 ? __ldcg(ws.nrm2 + pv) : (RZ ? ws.x_root_n2[g].x : 0.f);
+        }
+      }
+      if (!__all_sync(0xffffffffu, ready)) break;  // reported
+      const bool from_left = pv >= 0 && pv == v - 1 && r > 0;
+      const uint4* pb = pv >= 0 ? Z + pv * rs : (live && RZ ? RZ + (int64_t)g * rs : nullptr);
+      float2 n2, dot;
+      eight_rows_sums<true>(Z + (live ? v : 0) * rs, pb, live, from_left, sz.d, c, nx, ny, n2, dot);
+      if (live && c == 0 && GPO_BOUNDS(st, v, sz.N, kWhereStats)) {
+        ws.x_n2[v] = n2;
+        ws.x_dot[v] = pb ? dot : make_float2(0.f, 0.f);
+      }
+    }
+  }
+
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -448,11 +508,11 @@ cudaError_t setup_sim_tc() {
 }
 
 cudaError_t launch_sim_tc(const LaunchCtx& lc, const CUtensorMap& map, const gpo_batch& b, const Sizes& sz,
-                          const Ws& ws, const Params& p) {
+                          const Ws& ws, const Params& p, bool stats) {
   int grid = ws.max_items < lc.num_sms ? ws.max_items : lc.num_sms;
   if (grid < 1) return cudaSuccess;
-  sim_tc_kernel<<<grid, kThreads, sim_tc_smem_bytes(), lc.stream>>>(map, b.rollout_step_off, sz, ws, (float)p.kappa,
-                                                                      p.rule, p.debug_timeout);
+  sim_tc_kernel<<<grid, kThreads, sim_tc_smem_bytes(), lc.stream>>>(map, b, sz, ws, (float)p.kappa, p.rule, stats,
+                                                                      p.debug_timeout);
   return cudaGetLastError();
 }
 
