@@ -82,29 +82,54 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
   // each class's label is its smallest member.  Lock-free root unions (correct from any such
   // forest) finish the job if the rounds have not settled after kMaxRounds.
   // Items are dealt to warps (one item per warp at a time, lanes over its edges); the items'
-  // edge counts are read once into shared memory (X, free until the group math).
+  // edge counts are read once into shared memory (X, free until the group math), and the first
+  // round leaves the edges there too, if they fit, for the others (64 groups of 2048 states,
+  // whole call 490 -> 482 us with the loads ahead: three rounds over L2, one load at a time per
+  // lane, took 8.3 us).
   const int nit = ws.lab ? 0 : gi.nblk + gi.noff;  // the group's diagonal items, then its off-diagonal ones
   auto item_at = [&](int k) { return k < gi.nblk ? gi.blk0 + k : gi.off0 + (k - gi.nblk); };
   int* ecnt = reinterpret_cast<int*>(X);
   const bool cached = !tree && (size_t)nit * sizeof(int) <= group_scratch_bytes(n);
+  uint32_t* elist = reinterpret_cast<uint32_t*>(X) + nit;  // u | v << 16, group-local
+  const int ecap = cached ? (int)(group_scratch_bytes(n) / 4) - nit : 0;
+  __shared__ int s_ne;  // edges listed, or wanted
+  if (tid == 0) s_ne = 0;
   if (cached)
     for (int k = tid; k < nit; k += nt) ecnt[k] = min(ws.edge_count[item_at(k)], kEdgeCap);
   __syncthreads();
   const int lane = tid & 31, wid = tid >> 5, nwarp = nt >> 5;
   bool settled = ws.lab != nullptr;
+  int listed = -1;  // edges in elist, -1: not there
+  constexpr int kAhead = 4;  // an item's edges loaded ahead, per lane
   for (int round = 0; round < kMaxRounds && !settled; ++round) {
     int ch = 0;
-    for (int k = wid; k < nit; k += nwarp) {
-      const int ne = cached ? ecnt[k] : min(ws.edge_count[item_at(k)], kEdgeCap);
-      const int2* E = ws.edges + (size_t)item_at(k) * kEdgeCap;
-      for (int e = lane; e < ne; e += 32) {
-        const int2 uv = E[e];
-        const int u = uv.x - s0, v = uv.y - s0;
-        if ((unsigned)u < (unsigned)n && (unsigned)v < (unsigned)n) {
-          const int lu = lab[u], lv = lab[v];
-          if (lu != lv) {
-            atomicMin(&lab[max(lu, lv)], min(lu, lv));
-            ch = 1;
+    auto hook = [&](int u, int v) {
+      const int lu = lab[u], lv = lab[v];
+      if (lu != lv) {
+        atomicMin(&lab[max(lu, lv)], min(lu, lv));
+        ch = 1;
+      }
+    };
+    if (listed >= 0) {
+      for (int e = tid; e < listed; e += nt) hook((int)(elist[e] & 0xFFFFu), (int)(elist[e] >> 16));
+    } else {
+      for (int k = wid; k < nit; k += nwarp) {
+        const int ne = cached ? ecnt[k] : min(ws.edge_count[item_at(k)], kEdgeCap);
+        const int2* E = ws.edges + (size_t)item_at(k) * kEdgeCap;
+        int at = 0;
+        if (round == 0 && lane == 0) at = atomicAdd(&s_ne, ne);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        const bool list = round == 0 && at + ne <= ecap;
+        for (int e0 = lane; e0 < ne; e0 += 32 * kAhead) {
+          int2 uv[kAhead];  // all in flight before the first one's hook
+#pragma unroll
+          for (int i = 0; i < kAhead; ++i) uv[i] = e0 + 32 * i < ne ? __ldcg(&E[e0 + 32 * i]) : make_int2(s0, s0);
+#pragma unroll
+          for (int i = 0; i < kAhead; ++i) {
+            const int e = e0 + 32 * i, u = uv[i].x - s0, v = uv[i].y - s0;
+            const bool in = (unsigned)u < (unsigned)n && (unsigned)v < (unsigned)n;
+            if (list && e < ne) elist[at + e] = in ? (uint32_t)u | (uint32_t)v << 16 : 0u;  // (0, 0) links nothing
+            if (in) hook(u, v);
           }
         }
       }
@@ -117,6 +142,7 @@ __global__ void __launch_bounds__(1024) groups_kernel(gpo_batch b, gpo_outputs o
       }
     }
     settled = __syncthreads_or(ch) == 0;
+    if (round == 0 && s_ne <= ecap) listed = s_ne;
   }
   if (!settled) {
     for (int k = 0; k < nit; ++k) {
