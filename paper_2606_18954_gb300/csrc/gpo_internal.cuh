@@ -30,7 +30,6 @@ enum : int {
   kStError = 0,     // (words 0 and 1, one 64-bit value) the call's tag << 16 | first gpo_status reported
                     // by any kernel of the call; another tag: none
   kStItems = 2,     // number of similarity work items planned
-  kStTicket = 3,    // last-block ticket of the prep kernel
   kStDetail = 4,    // first failing index (debug aid)
   kStWhere = 5,     // kernel that reported the error (debug aid)
 };

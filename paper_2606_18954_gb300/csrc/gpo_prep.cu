@@ -51,8 +51,9 @@ __device__ int block_incl_scan(int x, int* warp_tot) {
 
 // ---------------------------------------------------------------------------
 // K0: validate the offset arrays, rewards and step lengths; write per-state
-// (rollout, depth) and per-rollout group; the last block to finish plans the
-// similarity work items.  Nothing is dereferenced before its range is checked.
+// (rollout, depth) and per-rollout group; every block plans its share of the
+// similarity work items (the last block to finish planned them all before: 10.5 of
+// 22 us for 5120 items).  Nothing is dereferenced before its range is checked.
 __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes sz, Ws ws) {
   const Status st{ws.status, ws.tag};
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -104,45 +105,45 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
     }
   }
 
-  // ---- last block: plan the work items
-  __shared__ int s_last;
+  // ---- plan the work items: every block counts all groups' items (the prefix sums below need
+  //      nothing but the offsets) and writes its share of them.  An error above, or in another
+  //      block, leaves the abort flag, at which the later kernels stop.
   __shared__ int s_warp[32];
-  __shared__ int s_carry;
   __shared__ int s_incl[kPlanThreads], s_s0[kPlanThreads], s_n[kPlanThreads];
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&st.p[kStTicket], 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  const bool ok = !aborted(st);
+  int carry = 0;  // items of the groups before `base`
   // items group by group: a group's diagonal items (one per row block, block order), then
   // its off-diagonal ones; every item an off-diagonal item waits for thus comes before it
   for (int base = 0; base < sz.G; base += kPlanThreads) {
     const int g = base + threadIdx.x;
     int cnt = 0, nb = 0, s0 = 0, n = 0;
-    if (ok && g < sz.G) {
+    if (g < sz.G) {
       const int r0 = go[g], r1 = go[g + 1];
-      s0 = tree ? b.group_state_off[g] : so[r0];
-      n = (tree ? b.group_state_off[g + 1] : so[r1]) - s0;
-      if (tree && (s0 < 0 || n < 0 || s0 + n > sz.N)) {  // reported by tree_prep_kernel
+      if (tree) {
+        s0 = b.group_state_off[g];
+        n = b.group_state_off[g + 1] - s0;
+      } else if (r0 >= 0 && r0 <= sz.R && r1 >= 0 && r1 <= sz.R) {
+        s0 = so[r0];
+        n = so[r1] - s0;
+      }
+      if (s0 < 0 || n < 0 || n > sz.N || s0 > sz.N - n) {  // reported where the offsets are checked
         s0 = 0;
         n = 0;
       }
-      if (n > sz.maxn || n > GPO_MAX_GROUP_STATES) report(st, GPO_ERR_UNSUPPORTED, 0, g);
+      if (n > sz.maxn || n > GPO_MAX_GROUP_STATES) {
+        if (blockIdx.x == 0) report(st, GPO_ERR_UNSUPPORTED, 0, g);
+        n = 0;
+      }
       nb = blocks_for(n);
       cnt = nb + offdiag_for(n);
     }
     const int incl = block_incl_scan(cnt, s_warp);
-    if (ok && g < sz.G) {
+    if (g < sz.G && blockIdx.x == 0) {
       GroupInfo gi;
       gi.s0 = s0;
       gi.n = n;
       gi.r0 = go[g];
       gi.nr = go[g + 1] - gi.r0;
-      gi.blk0 = s_carry + incl - cnt;
+      gi.blk0 = carry + incl - cnt;
       gi.nblk = nb;
       gi.off0 = gi.blk0 + nb;
       gi.noff = cnt - nb;
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
     s_n[threadIdx.x] = n;
     __syncthreads();
     const int batch = s_incl[kPlanThreads - 1];
-    for (int j = threadIdx.x; j < batch && ok; j += kPlanThreads) {
+    for (int j = tid; j < batch; j += nth) {
       int lo = 0, hi = kPlanThreads - 1;  // first t with s_incl[t] > j
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
@@ -161,8 +162,8 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
         else lo = mid + 1;
       }
       const int gn = s_n[lo], gs0 = s_s0[lo], gnb = blocks_for(gn);
-      int idx = j - (s_incl[lo] - gnb - offdiag_for(gn));  // item index within the group
-      const int k = s_carry + j;
+      int idx = j - (lo > 0 ? s_incl[lo - 1] : 0);  // item index within the group
+      const int k = carry + j;
       if (k >= ws.max_items) continue;
       Item it;
       it.group = base + lo;
@@ -185,14 +186,12 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
       ws.items[k] = it;
       ws.edge_count[k] = 0;
     }
-    __syncthreads();
-    if (threadIdx.x == kPlanThreads - 1) s_carry += incl;
-    __syncthreads();
+    carry += batch;
+    __syncthreads();  // s_* read above
   }
-  if (threadIdx.x == 0) {
-    const int total = s_carry;
-    if (total > ws.max_items) report(st, GPO_ERR_WORKSPACE, 0, total);
-    st.p[kStItems] = aborted(st) ? 0u : (uint32_t)total;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (carry > ws.max_items) report(st, GPO_ERR_WORKSPACE, 0, carry);
+    st.p[kStItems] = carry > ws.max_items ? 0u : (uint32_t)carry;
   }
 }
 
@@ -350,7 +349,7 @@ cudaError_t launch_tree_prep(const LaunchCtx& lc, const gpo_batch& b, const Size
 }
 
 cudaError_t launch_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws) {
-  const int64_t work = 32 * ((int64_t)sz.R + 1);  // a warp per rollout
+  const int64_t work = max(32 * ((int64_t)sz.R + 1), (int64_t)ws.max_items);  // a warp per rollout, a thread per item
   int blocks = (int)((work + kPlanThreads - 1) / kPlanThreads);
   blocks = blocks < 1 ? 1 : (blocks > 4 * lc.num_sms ? 4 * lc.num_sms : blocks);
   prep_kernel<<<blocks, kPlanThreads, 0, lc.stream>>>(b, sz, ws);
@@ -816,13 +815,13 @@ cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Si
 // one coalesced round trip and broadcast by shuffles; each span is written
 // with 16-byte stores in its aligned middle and scalar stores at the ends.
 
-__global__ void __launch_bounds__(256) tokens_kernel(gpo_batch b, gpo_outputs o, Sizes sz, Ws ws) {
+__global__ void __launch_bounds__(256) tokens_kernel(gpo_batch b, gpo_outputs o, Sizes sz, Ws ws, int per) {
   if (aborted(Status{ws.status, ws.tag})) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t base = warp * 32; base < sz.N; base += nwarps * 32) {
-    const int64_t v = base + lane;
+  for (int64_t base = warp * per; base < sz.N; base += nwarps * per) {
+    const int64_t v = lane < per ? base + lane : sz.N;
     int64_t ts = 0;
     int L = 0;
     float va = 0.f, vc = 0.f, ve = 0.f;
@@ -835,7 +834,7 @@ __global__ void __launch_bounds__(256) tokens_kernel(gpo_batch b, gpo_outputs o,
       if (o.adv_eff) ve = ws.e_eff[v];
       if (o.eff_mask) vm = ws.e_mask[v];
     }
-    const int cnt = (int)(sz.N - base < 32 ? sz.N - base : 32);
+    const int cnt = (int)min((int64_t)per, sz.N - base);
     for (int j = 0; j < cnt; ++j) {
       const int64_t s = __shfl_sync(0xffffffffu, ts, j);
       const int64_t e = s + __shfl_sync(0xffffffffu, L, j);
@@ -852,10 +851,16 @@ __global__ void __launch_bounds__(256) tokens_kernel(gpo_batch b, gpo_outputs o,
 cudaError_t launch_tokens(const LaunchCtx& lc, const gpo_batch& b, const gpo_outputs& o, const Sizes& sz,
                           const Ws& ws) {
   if (sz.T == 0 || sz.N == 0) return cudaSuccess;
-  int64_t blocks = (sz.N + 255) / 256;  // one warp per 32 edges
+  // `per` edges per warp, their metadata in one round trip: 32, fewer where that leaves the GPU
+  // without warps (an edge's spans take a warp's serial time: 16 k edges at 32 per warp, 64
+  // blocks, 16.4 us, at 4 10.2 us; 131 k edges at 32 32.8, at 8 26.6 us)
+  const int64_t warps = (int64_t)lc.num_sms * 8 * 8;  // eight blocks of eight warps per SM
+  int per = 32;
+  while (per > 4 && (sz.N + per - 1) / per < warps) per /= 2;
+  int64_t blocks = ((sz.N + per - 1) / per + 7) / 8;
   const int64_t cap = (int64_t)lc.num_sms * 8;
   if (blocks > cap) blocks = cap;
-  tokens_kernel<<<(unsigned)blocks, 256, 0, lc.stream>>>(b, o, sz, ws);
+  tokens_kernel<<<(unsigned)blocks, 256, 0, lc.stream>>>(b, o, sz, ws, per);
   return cudaGetLastError();
 }
 
