@@ -1,7 +1,7 @@
 // Fused group-resident path: the whole advantage construction for bf16
 // prompt groups of at most 384 states, persistent CTAs working through their
 // groups.  Two instances of the kernel body (gpo_fused_body.cuh): one for groups
-// of up to 384 states (512 threads, one CTA per SM, 160 KB tile ring, 512 TMEM
+// of up to 384 states (512 threads, one CTA per SM, 156 KB tile ring, 512 TMEM
 // columns) and one for groups of up to 128 states (256 threads, two CTAs per SM,
 // 76 KB ring, 128 TMEM columns), chosen by the batch's largest group.
 //
@@ -34,7 +34,7 @@ namespace fused_large {
 constexpr int kMaxN = kFusedMaxStates;  // 384
 constexpr int kThreads = 512;
 constexpr int kMinBlocks = 1;
-constexpr int kRingBytes = 160 * 1024;
+constexpr int kRingBytes = 156 * 1024;
 constexpr int kTmemCols = 512;
 #include "gpo_fused_body.cuh"
 }  // namespace fused_large

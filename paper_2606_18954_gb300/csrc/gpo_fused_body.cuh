@@ -15,6 +15,9 @@ constexpr int kEpiThreads = kThreads - 128;     // warps 4..: accumulator drain
 constexpr int kReps = kEpiThreads / 128;        // drain warps per accumulator lane quarter
 constexpr int kWarpEdges = 256;                 // linked pairs listed per epilogue warp and group
 constexpr int kEdgeList = kWarpEdges * (kEpiThreads / 32);
+// Groups of two passes wait for the second one's MMAs after draining the first: the token scatter
+// of the group before is put there (deferred_tokens).
+constexpr bool kDeferTokens = kMaxN > 2 * kTileM;
 constexpr int kBarGroup = 1;                    // named barrier of the group warps
 constexpr int kBarEpi = 2;                      // named barrier of the drain warps
 constexpr int kBarSetup = 3;                    // named barrier of warps 2 and 3 (early set-up)
@@ -134,6 +137,10 @@ struct __align__(16) GroupSmem {
   int overflow;          // some warp found more pairs than its part of elist holds
   int nstat[2];          // group_eta_stats: rows with a dot, rows with the norm alone (group_row_stats:
                          // the next block of 8 rows)
+  int put_off;           // scatter put off: states of the group, its first token,
+  int64_t dbase;
+  uint32_t dts[kDeferTokens ? kMaxN + 1 : 1];  // of each state relative to it (they follow one another),
+  float dval[kDeferTokens ? kMaxN : 1];        // and each state's advantage
   uint16_t slist[kMaxN]; // those rows: with a dot from the front, the norm alone from the end
   Plan plan;
   uint32_t elist[kEdgeList];  // linked pairs of the group, kWarpEdges per epilogue warp: i | j << 16
@@ -415,6 +422,32 @@ __device__ __forceinline__ void tree_setup(const gpo_batch& b, const Sizes& sz, 
   bar_group();
 }
 
+// A half-warp (hl = its lane) writes x to dst[ts, te), dst 16-byte aligned: whole 16-byte chunks,
+// then the at most 3 + 3 tokens of the partial first and last one (which neighbour other states'
+// tokens) with scalar stores.
+__device__ __forceinline__ void half_warp_span(float* dst, int64_t ts, int64_t te, float x, int hl) {
+  const int64_t qa = (ts + 3) >> 2, qb = te >> 2;
+  const int64_t h1 = qa <= qb ? 4 * qa : te;  // head [ts, h1)
+  const int64_t t0 = qa <= qb ? 4 * qb : te;  // tail [t0, te)
+  const int64_t tp = hl < 4 ? ts + hl : t0 + (hl - 4);
+  const float4 v = make_float4(x, x, x, x);
+  for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(dst)[c] = v;
+  if (hl < 4 ? tp < h1 : (hl < 8 && tp < te)) dst[tp] = x;
+}
+
+// The token scatter that the group before put off, by the drain warps (thread tid of them).
+__device__ __forceinline__ void deferred_tokens(const gpo_outputs& o, const Sizes& sz, const GroupSmem* gs, int tid,
+                                                const Status& st) {
+  const int64_t base = gs->dbase;
+  const int n = gs->put_off;
+#pragma unroll 1
+  for (int i = tid >> 4; i < n; i += kEpiThreads / 16) {
+    const int64_t ts = base + gs->dts[i], te = base + gs->dts[i + 1];
+    if (!GPO_BOUNDS(st, ts, sz.T, kWhereTokens) || !GPO_BOUNDS(st, te - 1, sz.T, kWhereTokens)) continue;
+    half_warp_span(o.adv, ts, te, gs->dval[i], tid & 15);
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     fused_kernel(const __grid_constant__ CUtensorMap zmap, const __grid_constant__ CUtensorMap zmap32, gpo_batch b,
                  gpo_outputs o, Sizes sz, Ws ws, Params p) {
@@ -452,6 +485,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     mbar_init(&ctl->drain, 1);
     fence_mbar_init();
     gs->nstat[0] = gs->nstat[1] = 0;
+    gs->put_off = 0;
     tma_prefetch_desc(&zmap);
     tma_prefetch_desc(&zmap32);
   }
@@ -710,6 +744,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         uint32_t* wlist = gs->elist + ew * kWarpEdges;
         int wcount = 0;                       // pairs this warp found in the group (warp-uniform)
         for (int pass = 0; pass < pl.npass; ++pass, ++u) {
+          if (kDeferTokens && gs->put_off && pass == pl.npass - 1) deferred_tokens(o, sz, gs, te, st);
           const bool got = mbar_wait(&ctl->tfull, (uint32_t)u & 1u, st, 25);
           if (bar_any<kBarEpi, kEpiThreads>(!got)) {
             fail = true;
@@ -870,6 +905,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         }
       }
       if (bar_any<kBarGroup, kGThreads>(fail)) break;
+      if (kDeferTokens && gt == 0) gs->put_off = 0;
 
       // ---- next-layer budgets of a branching group (gpo_layer_budget)
       if (valid && p.mode == 1) {
@@ -930,46 +966,70 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
                            [] { bar_group(); }, [](bool f) { return bar_any<kBarGroup, kGThreads>(f); },
                            o.group_eff ? o.group_eff + g : nullptr, o.group_eff_graph ? o.group_eff_graph + g : nullptr);
         }
-        // ---- every token of an edge carries the edge's advantage (Sec. 4.5).  State-major:
-        //      each half-warp takes a state, its 16 lanes write the whole 16-byte chunks of the
-        //      state's token span, then the at most 3 + 3 tokens of its partial first and last
-        //      chunk (which neighbour other states' tokens) with scalar stores.
+        // ---- every token of an edge carries the edge's advantage (Sec. 4.5), state-major, a
+        //      half-warp per state.  With a group to follow on this CTA it is put off to that
+        //      group's last wait for its MMAs: a group of two passes waits ~13 us for the second one
+        //      (320 states of 2 KB), the scatter is ~6.5 us of stores, and the next group starts that
+        //      much earlier (512 groups of 320 states 241 -> 231 us).  The drain warps do it: with
+        //      warps 2 and 3 as well, a second copy of the code, 128 groups of 256 states lose more
+        //      (51.3 -> 52.0) than these gain, and those two alone take longer than the wait (268).
+        //      Only in the instance whose groups can take two passes; the per-token components
+        //      go out at once.
         const bool more = o.adv_cor || o.adv_eff || o.eff_mask;
-        const int hl = gt & 15;
-#pragma unroll 1
-        for (int i = gt >> 4; i < n; i += kGThreads / 16) {
-          const int64_t ts = gs->tstart[i], te = ts + gs->slen[i];
-          const float x = gs->eadv[i];
-          const int64_t qa = (ts + 3) >> 2, qb = te >> 2;
-          const int64_t h1 = qa <= qb ? 4 * qa : te;  // head [ts, h1)
-          const int64_t t0 = qa <= qb ? 4 * qb : te;  // tail [t0, te)
-          const int64_t tp = hl < 4 ? ts + hl : t0 + (hl - 4);
-          const bool scal = hl < 4 ? tp < h1 : (hl < 8 && tp < te);
-          // (debug build) every store below lies in the state's span [ts, te)
-          if (!GPO_BOUNDS(st, ts, sz.T, kWhereTokens) || !GPO_BOUNDS(st, te - 1, sz.T, kWhereTokens)) continue;
-          {
-            const float4 v = make_float4(x, x, x, x);
-            for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv)[c] = v;
-            if (scal) o.adv[tp] = x;
+        bool later = false;
+        if (kDeferTokens && !more && g + (int64_t)gridDim.x < sz.g1) {
+          int r2, nr2, s2, n2;
+          later = group_active(b, sz, g + (int)gridDim.x, r2, nr2, s2, n2) &&
+                  gs->tstart[n - 1] + gs->slen[n - 1] - gs->tstart[0] <= 0xFFFFFFFFll;
+        }
+        if (later) {
+          const int64_t base = gs->tstart[0];
+          if (gt == 0) {
+            gs->dbase = base;
+            gs->put_off = n;
           }
-          if (more) {
-            if (o.adv_cor) {
-              const float y = gs->ecor[i];
-              const float4 v = make_float4(y, y, y, y);
-              for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv_cor)[c] = v;
-              if (scal) o.adv_cor[tp] = y;
+          for (int i = gt; i < n; i += kGThreads) {
+            gs->dts[i] = (uint32_t)(gs->tstart[i] - base);
+            gs->dval[i] = gs->eadv[i];
+            if (i == n - 1) gs->dts[n] = (uint32_t)(gs->tstart[i] + gs->slen[i] - base);
+          }
+        } else {
+          const int hl = gt & 15;
+#pragma unroll 1
+          for (int i = gt >> 4; i < n; i += kGThreads / 16) {
+            const int64_t ts = gs->tstart[i], te = ts + gs->slen[i];
+            const float x = gs->eadv[i];
+            const int64_t qa = (ts + 3) >> 2, qb = te >> 2;
+            const int64_t h1 = qa <= qb ? 4 * qa : te;  // head [ts, h1)
+            const int64_t t0 = qa <= qb ? 4 * qb : te;  // tail [t0, te)
+            const int64_t tp = hl < 4 ? ts + hl : t0 + (hl - 4);
+            const bool scal = hl < 4 ? tp < h1 : (hl < 8 && tp < te);
+            // (debug build) every store below lies in the state's span [ts, te)
+            if (!GPO_BOUNDS(st, ts, sz.T, kWhereTokens) || !GPO_BOUNDS(st, te - 1, sz.T, kWhereTokens)) continue;
+            {
+              const float4 v = make_float4(x, x, x, x);
+              for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv)[c] = v;
+              if (scal) o.adv[tp] = x;
             }
-            if (o.adv_eff) {
-              const float y = gs->eeff[i];
-              const float4 v = make_float4(y, y, y, y);
-              for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv_eff)[c] = v;
-              if (scal) o.adv_eff[tp] = y;
-            }
-            if (o.eff_mask) {
-              const uint8_t m = gs->emask[i];
-              const uint32_t v = 0x01010101u * m;
-              for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<uint32_t*>(o.eff_mask)[c] = v;
-              if (scal) o.eff_mask[tp] = m;
+            if (more) {
+              if (o.adv_cor) {
+                const float y = gs->ecor[i];
+                const float4 v = make_float4(y, y, y, y);
+                for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv_cor)[c] = v;
+                if (scal) o.adv_cor[tp] = y;
+              }
+              if (o.adv_eff) {
+                const float y = gs->eeff[i];
+                const float4 v = make_float4(y, y, y, y);
+                for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv_eff)[c] = v;
+                if (scal) o.adv_eff[tp] = y;
+              }
+              if (o.eff_mask) {
+                const uint8_t m = gs->emask[i];
+                const uint32_t v = 0x01010101u * m;
+                for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<uint32_t*>(o.eff_mask)[c] = v;
+                if (scal) o.eff_mask[tp] = m;
+              }
             }
           }
         }
