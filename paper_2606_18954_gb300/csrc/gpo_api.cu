@@ -1,7 +1,10 @@
 // Host implementation of the C ABI declared in include/graphpo.h: argument
 // checks, workspace layout, TMA descriptor encoding and the launch sequence
-//   prep (validate + plan) -> row stats -> similarity merge -> per-group
-//   advantages -> per-token scatter
+//   fused (the group-resident kernels; for rows of d <= 256 and more groups than CTAs the
+//   compensated statistics of the later groups first), or
+//   prep (validate + plan) -> row statistics (CUDA-core similarity only) -> similarity merge
+//   (on the tensor cores with the compensated statistics) -> per-group advantages -> per-token
+//   scatter
 // all on the caller's stream.  Nothing here allocates device memory.
 #include <atomic>
 #include <cmath>

@@ -196,10 +196,9 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
 }
 
 // The compensated row statistics that the group's eta's ask for (where group_row_stats has
-// not computed every row's; all group threads, one
-// state each: thread gt has state gt; need: eta(p(v), v) of that state is read).  The rows
-// are known only once the classes are, when they have just been streamed and lie in L2, and
-// they are few: 0.2 to 0.45 of a chain batch's states (a step whose score differs from its
+// not computed every row's; all group threads, one state each: thread gt has state gt; need:
+// eta(p(v), v) of that state is read).  The rows are known only once the classes are, when they
+// have just been streamed and lie in L2, and they are few: 0.2 to 0.45 of a chain batch's states (a step whose score differs from its
 // parent's, below a parent whose class has several edges), 0.85 of a branching one's.  Two
 // lists, the rows with a dot (|z_v|^2 and <z_{p(v)}, z_v>) from the front of slist and the
 // parents that need |z|^2 alone from its end; a half-warp per row (half_warp_row_sums,
@@ -207,7 +206,8 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
 // and dependent sums at 14 warps per SM (a third of the issue slots used).  Results as float
 // pairs: |z|^2 in (rn, thr), free once the pairs are tested, the dot in (ecor, eeff).
 // Whole call, against the statistics of all rows (a CTA's first group while it streams in,
-// the groups after it in a launch of their own before): 512 groups of 320 states 273 -> 245 us.
+// the groups after it in a launch of their own before): 512 groups of 320 states 273 -> 245 us
+// (231 with the steps since).
 template <class Par>
 __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
                                                 int g, int s0, int n, bool need, Par par, int gt, int wg, int lane,
