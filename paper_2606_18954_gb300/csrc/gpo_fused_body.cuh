@@ -207,7 +207,7 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
 // pairs: |z|^2 in (rn, thr), free once the pairs are tested, the dot in (ecor, eeff).
 // Whole call, against the statistics of all rows (a CTA's first group while it streams in,
 // the groups after it in a launch of their own before): 512 groups of 320 states 273 -> 245 us
-// (231 with the steps since).
+// (223 with the steps since).
 template <class Par>
 __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
                                                 int g, int s0, int n, bool need, Par par, int gt, int wg, int lane,
@@ -431,7 +431,7 @@ __device__ __forceinline__ void half_warp_span(float* dst, int64_t ts, int64_t t
   const int64_t t0 = qa <= qb ? 4 * qb : te;  // tail [t0, te)
   const int64_t tp = hl < 4 ? ts + hl : t0 + (hl - 4);
   const float4 v = make_float4(x, x, x, x);
-  for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(dst)[c] = v;
+  for (int64_t c = qa + hl; c < qb; c += 16) __stcs(reinterpret_cast<float4*>(dst) + c, v);
   if (hl < 4 ? tp < h1 : (hl < 8 && tp < te)) dst[tp] = x;
 }
 
@@ -511,9 +511,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     int head = 0;
     uint32_t seq = 0, oldest = 0;  // slices issued; oldest slice not yet seen consumed
     bool ok = true;
-    // L2 policy: pass 0 of a two-pass group keeps its rows (pass 1 reads them again),
-    // pass 1 drops them first (their last read)
-    const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
+    // L2 policy: pass 0 of a two-pass group keeps its rows, which pass 1 reads again; the others have
+    // none, since group_eta_stats reads the rows after the last pass.  (Evict-first on pass 1 made
+    // those reads go to DRAM: 512 groups of 320 states read 557 MB for 337 MB of rows and took
+    // 231 us, 224 without it.)
+    const uint64_t keep = l2_policy_evict_last();
     for (int g = sz.g0 + (int)blockIdx.x; g < sz.g1 && ok; g += gridDim.x) {
       int r0, nr, s0, n;
       if (!group_active(b, sz, g, r0, nr, s0, n)) continue;
@@ -522,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       for (int pass = 0; pass < npass && ok; ++pass) {
         const int row0 = npass == 2 && pass == 0 ? kTileM : 0;  // pass 0 of two never reads block 0
         const int bytes = (rows - row0) * 128;
-        const int hint = npass == 1 ? 0 : (pass == 0 ? 1 : 2);
+        const bool again = npass == 2 && pass == 0;  // pass 1 reads these rows again
         for (int k = 0; k < KT && ok; ++k) {
           const int off = ring_place(head, bytes);
           while (oldest < seq) {
@@ -542,11 +544,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           mbar_arrive_expect_tx(&ctl->full[bi], (uint32_t)bytes);
           for (int r = row0; r < rows;) {  // 128-row boxes, then 32-row boxes for the tail
             const bool big = rows - r >= kTileM;
-            if (hint == 0)
-              tma_load_2d(t + (r - row0) * 128, big ? &zmap : &zmap32, &ctl->full[bi], k * kTileK, s0 + r);
+            if (again)
+              tma_load_2d_hint(t + (r - row0) * 128, big ? &zmap : &zmap32, &ctl->full[bi], k * kTileK, s0 + r, keep);
             else
-              tma_load_2d_hint(t + (r - row0) * 128, big ? &zmap : &zmap32, &ctl->full[bi], k * kTileK, s0 + r,
-                               hint == 1 ? keep : drop);
+              tma_load_2d(t + (r - row0) * 128, big ? &zmap : &zmap32, &ctl->full[bi], k * kTileK, s0 + r);
             r += big ? kTileM : kTailRows;
           }
           ctl->slice_off[bi] = off;
@@ -974,7 +975,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         //      warps 2 and 3 as well, a second copy of the code, 128 groups of 256 states lose more
         //      (51.3 -> 52.0) than these gain, and those two alone take longer than the wait (268).
         //      Only in the instance whose groups can take two passes; the per-token components
-        //      go out at once.
+        //      go out at once.  Streaming stores: they take no place in L2 from the rows that are
+        //      still to be read (256 groups of 56 states with every output 53.4 -> 49.8 us).
         const bool more = o.adv_cor || o.adv_eff || o.eff_mask;
         bool later = false;
         if (kDeferTokens && !more && g + (int64_t)gridDim.x < sz.g1) {
@@ -1008,26 +1010,26 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
             if (!GPO_BOUNDS(st, ts, sz.T, kWhereTokens) || !GPO_BOUNDS(st, te - 1, sz.T, kWhereTokens)) continue;
             {
               const float4 v = make_float4(x, x, x, x);
-              for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv)[c] = v;
+              for (int64_t c = qa + hl; c < qb; c += 16) __stcs(reinterpret_cast<float4*>(o.adv) + c, v);
               if (scal) o.adv[tp] = x;
             }
             if (more) {
               if (o.adv_cor) {
                 const float y = gs->ecor[i];
                 const float4 v = make_float4(y, y, y, y);
-                for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv_cor)[c] = v;
+                for (int64_t c = qa + hl; c < qb; c += 16) __stcs(reinterpret_cast<float4*>(o.adv_cor) + c, v);
                 if (scal) o.adv_cor[tp] = y;
               }
               if (o.adv_eff) {
                 const float y = gs->eeff[i];
                 const float4 v = make_float4(y, y, y, y);
-                for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<float4*>(o.adv_eff)[c] = v;
+                for (int64_t c = qa + hl; c < qb; c += 16) __stcs(reinterpret_cast<float4*>(o.adv_eff) + c, v);
                 if (scal) o.adv_eff[tp] = y;
               }
               if (o.eff_mask) {
                 const uint8_t m = gs->emask[i];
                 const uint32_t v = 0x01010101u * m;
-                for (int64_t c = qa + hl; c < qb; c += 16) reinterpret_cast<uint32_t*>(o.eff_mask)[c] = v;
+                for (int64_t c = qa + hl; c < qb; c += 16) __stcs(reinterpret_cast<uint32_t*>(o.eff_mask) + c, v);
                 if (scal) o.eff_mask[tp] = m;
               }
             }
