@@ -26,8 +26,6 @@ struct gpo_ctx {
   int num_sms;
   uint32_t* host_status;      // pinned copy of the workspace status words
   const uint32_t* last_status; // device status words of the last gpo_compute
-  uint64_t tag;                // tag of the errors of the calls since the last clearing one (see Status)
-  uint64_t last_tag;           // tag of last_status
   char msg[512];
   bool timing;
   int nstages;                 // stages recorded by the last gpo_compute
@@ -254,7 +252,6 @@ gpo_status gpo_create(gpo_ctx** out, const gpo_params* params) {
   if (!c) return GPO_ERR_CUDA;
   c->params = *params;
   c->last_status = nullptr;
-  c->tag = c->last_tag = kClearedTag;
   c->msg[0] = 0;
   cudaDeviceProp prop;
   if (cudaGetDevice(&c->device) != cudaSuccess || cudaGetDeviceProperties(&prop, c->device) != cudaSuccess) {
@@ -316,7 +313,7 @@ gpo_status gpo_workspace_size(const gpo_ctx* ctx, const gpo_batch* batch, size_t
 
 namespace {
 
-// A tag that no other call of this process has (48 bits, never 0 or kClearedTag): a counter
+// A tag that no other call of this process has (48 bits, never 0): a counter
 // passed through the finaliser of SplitMix64 (Steele, Lea, Flood 2014), a bijection of 64 bits,
 // of which the top 48 are kept, so that small integers or text in memory never look like one.
 uint64_t fresh_tag() {
@@ -326,7 +323,7 @@ uint64_t fresh_tag() {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     z = (z ^ (z >> 31)) >> 16;
-    if (z > kClearedTag) return z;
+    if (z != 0) return z;
   }
 }
 
@@ -337,9 +334,9 @@ struct BudgetReq {
   int32_t* budget;
 };
 
-// What a call does with the status words first: nothing (its errors join those of the calls
-// since the last clearing one), clear them, or, where that saves the clearing, take a tag of
-// its own (kFresh: a whole call, with no later ranges that another context might add).
+// What a call does with the status words first: nothing (its errors join those that the words
+// hold), clear them, or, where that saves the clearing, sign them with a tag of its own
+// (kFresh: a whole call).
 enum class StatusInit { kKeep, kClear, kFresh };
 
 // The path for groups [g0, g1) of the batch.
@@ -444,22 +441,18 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   };
   cudaError_t e = cudaSuccess;
   if (ctx->timing) e = cudaEventRecord(ctx->ev[0], lc.stream);
-  // A fresh tag instead of a memset for the one-kernel paths (the tiled path's planning words
-  // start from zero), but not in a graph, whose replays would share it
+  // A fresh tag instead of a memset for the one-kernel paths (the tiled path's kernels do not
+  // sign the words), but not in a graph, whose replays would share it
   if (init == StatusInit::kFresh) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (!(fused || fused32) || cudaStreamIsCapturing(lc.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
       cudaGetLastError();  // (the legacy stream beside a capture: the memset reports it)
       init = StatusInit::kClear;
-    } else {
-      ctx->tag = fresh_tag();
     }
   }
-  if (init == StatusInit::kClear) {
-    ctx->tag = kClearedTag;
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws.status, 0, sizeof(uint32_t) * kStatusWords, lc.stream);
-  }
-  ws.tag = ctx->tag;
+  ws.tag = init == StatusInit::kFresh ? fresh_tag() : (init == StatusInit::kClear ? 0 : kStoredTag);
+  if (init == StatusInit::kClear && e == cudaSuccess)
+    e = cudaMemsetAsync(ws.status, 0, sizeof(uint32_t) * kStatusWords, lc.stream);
   if (g1 <= g0) {
     // nothing to compute (a call that only clears the status words)
   } else if (fused32) {
@@ -501,7 +494,6 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   }
   ctx->nstages = ns;
   ctx->last_status = ws.status;
-  ctx->last_tag = ws.tag;
   if (e != cudaSuccess) return set_msg(ctx, "launch failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
   return GPO_OK;
 }
@@ -797,7 +789,6 @@ gpo_status gpo_loss_plan(gpo_ctx* ctx, const gpo_batch* batch, void* plan, size_
   if (e == cudaSuccess) e = launch_loss_plan(lc, *batch, loss_sizes(*batch), lp);
   ctx->nstages = 0;
   ctx->last_status = lp.status;
-  ctx->last_tag = kClearedTag;
   if (e != cudaSuccess) return set_msg(ctx, "launch failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
   return GPO_OK;
 }
@@ -864,7 +855,6 @@ gpo_status gpo_token_loss(gpo_ctx* ctx, const gpo_batch* batch, void* plan, cons
   }
   ctx->nstages = ns;
   ctx->last_status = lp.status;
-  ctx->last_tag = kClearedTag;
   if (e != cudaSuccess) return set_msg(ctx, "launch failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
   return GPO_OK;
 }
@@ -899,8 +889,8 @@ gpo_status gpo_sync_status(gpo_ctx* ctx, void* stream) {
   if (!ctx->last_status) return GPO_OK;
   e = cudaMemcpy(ctx->host_status, ctx->last_status, sizeof(uint32_t) * kStatusWords, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return set_msg(ctx, "status read failed: %s", cudaGetErrorString(e)), GPO_ERR_CUDA;
-  const uint64_t word = (uint64_t)ctx->host_status[kStError + 1] << 32 | ctx->host_status[kStError];
-  const uint32_t code = word >> 16 == ctx->last_tag ? (uint32_t)(word & 0xFFFFu) : 0u;
+  auto word = [&](int i) { return (uint64_t)ctx->host_status[i + 1] << 32 | ctx->host_status[i]; };
+  const uint32_t code = is_error(word(kStError), word(kStTag)) ? (uint32_t)(word(kStError) & 0xFFFFu) : 0u;
   if (code != 0)
     set_msg(ctx, "%s (kernel %u, index %u)", gpo_status_string((gpo_status)code), ctx->host_status[kStWhere],
             ctx->host_status[kStDetail]);

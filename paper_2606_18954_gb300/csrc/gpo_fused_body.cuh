@@ -466,6 +466,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
 
   const bool tree = b.parent != nullptr;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    sign_status(st);
     if (b.group_rollout_off[0] != 0 || b.group_rollout_off[sz.G] != sz.R) report(st, GPO_ERR_SHAPE, 2, 0);
     if (tree) {
       if (b.group_state_off[0] != 0 || b.group_state_off[sz.G] != sz.N) report(st, GPO_ERR_SHAPE, 2, 1);

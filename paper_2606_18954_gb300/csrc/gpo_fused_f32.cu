@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(NT, 1) fused_f32_kernel(gpo_batch b, gpo_outpu
   float* part = Zs + (size_t)sz.maxn * ds;  // Gram partial sums of parts 1.. (f32_partial_bytes)
   const float kappa = p.kappa_f;
   if (blockIdx.x == 0 && tid == 0) {
+    sign_status(st);
     if (b.group_rollout_off[0] != 0 || b.group_rollout_off[sz.G] != sz.R) report(st, GPO_ERR_SHAPE, 2, 0);
     if (b.rollout_step_off[0] != 0 || b.rollout_step_off[sz.R] != sz.N) report(st, GPO_ERR_SHAPE, 2, 1);
     if (b.rollout_token_off[0] != 0 || b.rollout_token_off[sz.R] != sz.T) report(st, GPO_ERR_SHAPE, 2, 2);

@@ -27,11 +27,13 @@ constexpr int64_t kPipeMinChunkBytes = (int64_t)8 << 20;
 
 // status words (uint32) at the head of the workspace
 enum : int {
-  kStError = 0,     // (words 0 and 1, one 64-bit value) the call's tag << 16 | first gpo_status reported
-                    // by any kernel of the call; another tag: none
+  kStError = 0,     // (words 0 and 1, one 64-bit value) tag << 16 | first gpo_status reported by any
+                    // kernel since the words were cleared or signed; a tag other than kStTag's: none
   kStItems = 2,     // number of similarity work items planned
   kStDetail = 4,    // first failing index (debug aid)
   kStWhere = 5,     // kernel that reported the error (debug aid)
+  kStTag = 6,       // (words 6 and 7) the tag in force: 0 once the words are cleared, else that of the
+                    // whole call that signed them
 };
 
 // A similarity work item: rows [row0, row0+128) of one prompt group against
@@ -50,7 +52,8 @@ struct GroupInfo {
 // Device pointers into the caller's workspace (computed on the host).
 struct Ws {
   uint32_t* status;      // [kStatusWords]
-  uint64_t tag;          // the call's tag in the status words (see Status)
+  uint64_t tag;          // 0: the words were cleared before the kernel; kStoredTag: the tag in kStTag;
+                         // else the call's own tag, with which its kernel signs the words (see Status)
   Item* items;           // [max_items]: per group, its diagonal items, then its off-diagonal ones
   int* blk_ready;        // [max_items]: at a diagonal item's position, set once it has written its norms
   GroupInfo* groups;     // [G]
@@ -103,25 +106,43 @@ struct Params {
 
 // ------------------------------------------------------------------ errors
 
-// The status words of a call.  An error carries the call's 48-bit tag, so that words left by
-// earlier calls, or never written, are no error of this one: a call with a tag of its own
-// (fresh_tag on the host) needs no clearing of the words first, which as a memset node before
-// the kernel cost every call about 2 us.  Calls whose words are cleared share kClearedTag.
+// The status words of a workspace.  An error counts when its 48-bit tag is the one in force,
+// kStTag: a whole call with a tag of its own (fresh_tag on the host) signs the words with it
+// (sign_status), so that words left by earlier calls, or never written, are no error, and needs
+// no clearing of them first, which as a memset node before the kernel cost every call about
+// 2 us.  Where the words are cleared the tag in force is 0, and so is that of the calls that
+// clear them; a call that adds to the words takes the tag that it finds there.  Which errors
+// count is thus the workspace's state alone: contexts, streams and replayed graphs that use
+// it in turn agree on it.
 struct Status {
   uint32_t* p;
-  uint64_t tag;
+  uint64_t tag;  // as Ws::tag
 };
-constexpr uint64_t kClearedTag = 1;
+constexpr uint64_t kStoredTag = ~0ull;  // (no tag: tags have 48 bits)
+
+__device__ __forceinline__ uint64_t status_tag(const Status& st) {
+  return st.tag == kStoredTag ? *reinterpret_cast<volatile const uint64_t*>(st.p + kStTag) : st.tag;
+}
+// Whether the error word holds an error with the tag t.
+__host__ __device__ __forceinline__ bool is_error(uint64_t word, uint64_t t) {
+  return (word & 0xFFFFu) != 0 && word >> 16 == t;
+}
+
+// By one thread of a call's last kernel, before it reports anything (the kernels before it
+// carry the same tag; whoever reads the words comes after the call).
+__device__ __forceinline__ void sign_status(const Status& st) {
+  if (st.tag != 0 && st.tag != kStoredTag) *reinterpret_cast<volatile uint64_t*>(st.p + kStTag) = st.tag;
+}
 
 __device__ __forceinline__ bool aborted(const Status& st) {
-  return *reinterpret_cast<volatile const uint64_t*>(st.p + kStError) >> 16 == st.tag;
+  return is_error(*reinterpret_cast<volatile const uint64_t*>(st.p + kStError), status_tag(st));
 }
 
 __device__ __forceinline__ void report(const Status& st, int code, int where, int detail) {
   unsigned long long* w = reinterpret_cast<unsigned long long*>(st.p + kStError);
-  const unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(w);
-  if (old >> 16 == st.tag) return;  // not the call's first error
-  if (atomicCAS(w, old, (unsigned long long)st.tag << 16 | (unsigned)code) == old) {
+  const unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(w), t = status_tag(st);
+  if (is_error(old, t)) return;  // not the first error
+  if (atomicCAS(w, old, t << 16 | (unsigned)code) == old) {
     st.p[kStWhere] = (uint32_t)where;
     st.p[kStDetail] = (uint32_t)detail;
   }

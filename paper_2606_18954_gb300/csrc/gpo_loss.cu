@@ -61,7 +61,7 @@ __device__ __forceinline__ int64_t segment_starts(const int32_t* step_len, int v
 }
 
 __global__ void __launch_bounds__(kPlanThreads) loss_plan_kernel(gpo_batch b, Sizes sz, LossPlan lp) {
-  const Status st{lp.status, kClearedTag};
+  const Status st{lp.status, 0};
   const int g = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const bool tree = b.parent != nullptr;
   const int32_t* go = b.group_rollout_off;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kPlanThreads) loss_plan_kernel(gpo_batch b, Si
 }
 
 __global__ void __launch_bounds__(256) loss_weights_kernel(Sizes sz, LossPlan lp) {
-  if (aborted(Status{lp.status, kClearedTag})) return;
+  if (aborted(Status{lp.status, 0})) return;
   const double groups = (double)lp.status[kLossWordGroups];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < sz.N; v += stride) {
@@ -352,9 +352,9 @@ template <bool kSplit, bool kKL>
 __global__ void __launch_bounds__(kLossThreads, kKL ? 3 : 4) token_loss_kernel(LossArgs a, LossPlan lp) {
   extern __shared__ __align__(16) unsigned char loss_smem[];
   LossSmem<kSplit, kKL>& sm = *reinterpret_cast<LossSmem<kSplit, kKL>*>(loss_smem);
-  if (aborted(Status{lp.status, kClearedTag})) return;  // the plan found a layout error (read before any block ran)
+  if (aborted(Status{lp.status, 0})) return;  // the plan found a layout error (read before any block ran)
   if (lp.dims[0] != a.N || lp.dims[1] != a.T) {  // a plan of another batch shape
-    if (threadIdx.x == 0) report(Status{lp.status, kClearedTag}, GPO_ERR_SHAPE, 7, 0);
+    if (threadIdx.x == 0) report(Status{lp.status, 0}, GPO_ERR_SHAPE, 7, 0);
     return;
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -19,9 +19,9 @@
 // from a new primary context after cudaDeviceReset, never receives an address
 // that belongs to a different context.  Make the first call in each context
 // before any stream capture.  Every later call in the same context reuses the
-// same array, which keeps whatever the previous call left in it: the status
-// words at its head are cleared by each call, and every other part of the
-// workspace is written before it is read.  Calls in one context whose work
+// same array, which keeps whatever the previous call left in it: each call
+// clears the status words at its head or signs them with a tag of its own, and
+// every other part of the workspace is written before it is read.  Calls in one context whose work
 // overlaps on the GPU (other streams, other host threads) share the array and
 // race; the caller must order them.
 #include <cstdio>

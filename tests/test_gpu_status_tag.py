@@ -87,3 +87,93 @@ def test_ranges_after_a_whole_call(gp_mod):
     db.reward.copy_(good)
     gp.compute_into(db, out)
     gp.check()
+
+
+def other_work(P, gp, kind):
+    """A whole call of another batch in a workspace of its own, on a one-kernel path."""
+    import torch
+    from paper_2606_18954_gb300 import workloads as W
+    b = W.make_tree_batch(W.TREE_CONFIGS["tree"].scaled(2)) if kind == "budget" else batch_of("math", 2)
+    db = P.Batch.from_arrays(b, device="cuda")
+    ws = torch.empty(gp.workspace_size(db), dtype=torch.uint8, device="cuda")
+    if kind == "budget":
+        gp.layer_budget(db, 2, 2, workspace=ws)
+    else:
+        gp.compute_into(db, gp.alloc_outputs(db), workspace=ws)
+
+
+@pytest.mark.parametrize("kind", ["compute", "budget"])
+def test_ranges_around_a_call_elsewhere(gp_mod, kind):
+    """A workspace's ranges share their first error whatever the context does elsewhere between."""
+    import torch
+    b, p, gp, db, out = setup(gp_mod, "math", 4)
+    ws, stream = gp.workspace(db), torch.cuda.current_stream()
+    good, length = db.reward.clone(), db.step_len.clone()
+    db.reward[0] = 7    # group 0: GPO_ERR_BAD_REWARD
+    db.step_len[-1] = 0  # group 3: GPO_ERR_SHAPE
+    gp.compute_groups(db, out, 0, 1, True, ws, stream)
+    other_work(gp_mod, gp, kind)
+    gp.compute_groups(db, out, 2, 2, False, ws, stream)
+    with pytest.raises(gp_mod.GraphPOError) as e:
+        gp.check()
+    assert e.value.code == 3  # the first range's
+    db.reward.copy_(good)
+    db.step_len.copy_(length)
+    gp.compute_groups(db, out, 0, 2, True, ws, stream)
+    other_work(gp_mod, gp, kind)
+    gp.compute_groups(db, out, 2, 2, False, ws, stream)
+    gp.check()
+    compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, p), kind)
+
+
+def test_ranges_of_two_contexts(gp_mod):
+    """Two contexts that add ranges to one workspace, one of them after a whole call of its own."""
+    import torch
+    _, _, gp, db, out = setup(gp_mod, "math", 4)
+    gp2 = setup(gp_mod, "math", 2)[2]
+    other_work(gp_mod, gp2, "compute")
+    ws, stream = gp.workspace(db), torch.cuda.current_stream()
+    db.reward[0] = 7
+    db.step_len[-1] = 0
+    gp.compute_groups(db, out, 0, 1, True, ws, stream)
+    gp2.compute_groups(db, out, 1, 3, False, ws, stream)
+    for g in (gp, gp2):
+        with pytest.raises(gp_mod.GraphPOError) as e:
+            g.check()
+        assert e.value.code == 3
+    db.reward[0] = 0
+    gp.compute_groups(db, out, 0, 1, True, ws, stream)
+    gp2.compute_groups(db, out, 1, 3, False, ws, stream)
+    for g in (gp, gp2):  # the second context's error
+        with pytest.raises(gp_mod.GraphPOError) as e:
+            g.check()
+        assert e.value.code == 2
+
+
+@pytest.mark.parametrize("name,groups", NAMES)
+def test_replays_after_an_eager_call(gp_mod, name, groups):
+    import torch
+    b, p, gp, db, out = setup(gp_mod, name, groups)
+    gp.compute_into(db, out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gp.compute_into(db, out)
+    good = db.reward.clone()
+    for _ in range(2):
+        db.reward.copy_(good)
+        gp.compute_into(db, out)  # eager, same context and workspace
+        db.reward[0] = 7
+        graph.replay()
+        with pytest.raises(gp_mod.GraphPOError) as e:
+            gp.check()
+        assert e.value.code == 3
+        db.reward.copy_(good)
+        gp.compute_into(db, out)
+        gp.check()
+        db.reward[0] = 7
+        gp.compute_into(db, out)
+        db.reward.copy_(good)
+        out["adv"].zero_()
+        graph.replay()
+        gp.check()
+        compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, p), f"{name} replay")
