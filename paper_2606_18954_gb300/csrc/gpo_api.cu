@@ -19,6 +19,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "gpo_internal.cuh"
+#include "gpo_tag.cuh"
 
 struct gpo_ctx {
   gpo_params params;
@@ -313,17 +314,12 @@ gpo_status gpo_workspace_size(const gpo_ctx* ctx, const gpo_batch* batch, size_t
 
 namespace {
 
-// A tag that no other call of this process has (48 bits, never 0): a counter
-// passed through the finaliser of SplitMix64 (Steele, Lea, Flood 2014), a bijection of 64 bits,
-// of which the top 48 are kept, so that small integers or text in memory never look like one.
+// A tag that no other call of this process has.
 uint64_t fresh_tag() {
   static std::atomic<uint64_t> calls{0};
   while (true) {
-    uint64_t z = calls.fetch_add(1, std::memory_order_relaxed) * 0x9E3779B97F4A7C15ull + 0x2545F4914F6CDD1Dull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    z = (z ^ (z >> 31)) >> 16;
-    if (z != 0) return z;
+    const uint64_t t = tag_of(calls.fetch_add(1, std::memory_order_relaxed));
+    if (t != 0) return t;
   }
 }
 
