@@ -12,9 +12,12 @@
 // the diagonal of its Gram tile (for the threshold test; eta uses the compensated
 // statistics), writes them to the workspace and raises the block's ready flag; an off-diagonal
 // item waits (bounded) for the flags of its row and column blocks before its
-// epilogue reads them.  Every wait is on an item earlier in the list, diagonal items
-// never wait, and each CTA takes its items in list order, so every wait ends.
-// Persistent CTAs (one per SM) walk the item list.
+// epilogue reads them, and the statistics warps wait for those of their rows.  Every wait
+// is on a diagonal item, which waits for nothing, of this or another CTA, and each CTA takes
+// its items in list order; the launch is cooperative, so that all CTAs are resident before
+// any of them waits (an ordinary one beside another stream's kernel can leave a CTA whose
+// flag the resident ones wait for without an SM until they give up).  So every wait ends.
+// Persistent CTAs (at most one per SM) walk the item list.
 // Warp roles:
 //   warp 0 (one lane)  TMA producer: 128-row boxes of Z, 64 bf16 wide, 128B swizzle
 //   warp 1 (one lane)  MMA issuer: D[128 x N] += A[128 x 64] * B[N x 64]^T per k-step,
@@ -511,9 +514,23 @@ cudaError_t launch_sim_tc(const LaunchCtx& lc, const CUtensorMap& map, const gpo
                           const Ws& ws, const Params& p, bool stats) {
   int grid = ws.max_items < lc.num_sms ? ws.max_items : lc.num_sms;
   if (grid < 1) return cudaSuccess;
-  sim_tc_kernel<<<grid, kThreads, sim_tc_smem_bytes(), lc.stream>>>(map, b, sz, ws, (float)p.kappa, p.rule, stats,
-                                                                      p.debug_timeout);
-  return cudaGetLastError();
+  cudaLaunchAttribute coop;
+  coop.id = cudaLaunchAttributeCooperative;
+  coop.val.cooperative = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = sim_tc_smem_bytes();
+  cfg.stream = lc.stream;
+  cfg.attrs = &coop;
+  cfg.numAttrs = 1;
+  // a stream confined to part of the SMs holds fewer CTAs: any number of them does the work
+  for (;; grid = (grid + 1) / 2) {
+    cfg.gridDim = dim3((unsigned)grid);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, sim_tc_kernel, map, b, sz, ws, (float)p.kappa, p.rule, (int)stats,
+                                             p.debug_timeout);
+    if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1) return e;
+    cudaGetLastError();
+  }
 }
 
 }  // namespace gpo
