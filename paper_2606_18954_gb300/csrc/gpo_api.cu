@@ -476,7 +476,7 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
       const bool exact_first = !use_tc && !bud && b.emb_dtype == GPO_EMB_F32;
       auto exact = [&] { return launch_exact_stats(lc, b, sz, ws, true); };
       if (use_tc) {
-        if (b.root_emb && !bud) e = stage("root_norms", [&] { return launch_root_norms(lc, b, sz, ws); });
+        if (b.root_emb && !bud) e = stage("root_norms", [&] { return launch_root_norms(lc, b, sz, ws, true); });
         if (e == cudaSuccess) e = stage("similarity", [&] { return launch_sim_tc(lc, map, b, sz, ws, pp, !bud); });
       } else {
         if (exact_first) e = stage("exact_stats", exact);

@@ -29,11 +29,13 @@ constexpr int64_t kPipeMinChunkBytes = (int64_t)8 << 20;
 enum : int {
   kStError = 0,     // (words 0 and 1, one 64-bit value) tag << 16 | first gpo_status reported by any
                     // kernel since the words were cleared or signed; a tag other than kStTag's: none
-  kStItems = 2,     // number of similarity work items planned
+  kStItems = 2,     // number of similarity work items planned, or kPlanFault
   kStDetail = 4,    // first failing index (debug aid)
   kStWhere = 5,     // kernel that reported the error (debug aid)
   kStTag = 6,       // (words 6 and 7) the tag in force: 0 once the words are cleared, else that of the
                     // whole call that signed them
+  kStPlan = 8,      // with kPlanFault: the status to report,
+  kStPlanIndex = 9, // and the index it is about
 };
 
 // A similarity work item: rows [row0, row0+128) of one prompt group against
@@ -146,6 +148,19 @@ __device__ __forceinline__ void report(const Status& st, int code, int where, in
     st.p[kStWhere] = (uint32_t)where;
     st.p[kStDetail] = (uint32_t)detail;
   }
+}
+
+// A fault of the tiled path's plan alone (a group above the limit, too many items) counts only
+// where every check of the layout has passed, which the prep kernel's blocks do not know of
+// each other: it leaves kPlanFault for the number of items, and the kernels after it, before
+// an error of their own and in place of any work, report the fault here (unless an error is
+// there).  Returns whether there was one.
+constexpr int kPlanFault = -1;
+__device__ __forceinline__ bool plan_fault(const Status& st) {
+  const volatile uint32_t* w = st.p;
+  if ((int)w[kStItems] != kPlanFault) return false;
+  report(st, (int)w[kStPlan], 0, (int)w[kStPlanIndex]);
+  return true;
 }
 
 // Bounds checks of the debug build (-DGPO_DEBUG, a stand-in for a device memory checker):
@@ -852,8 +867,9 @@ cudaError_t launch_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz
 // with_norms: ws.nrm2 holds every row's fp32 squared norm (the similarity stage ran first)
 cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                                bool with_norms = false);
-// |prompt embedding|^2 of groups [g0, g1) into ws.x_root_n2 (bf16)
-cudaError_t launch_root_norms(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
+// |prompt embedding|^2 of groups [g0, g1) into ws.x_root_n2 (bf16); after_prep: the prep kernel ran
+cudaError_t launch_root_norms(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
+                              bool after_prep);
 cudaError_t launch_tree_prep(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);
 cudaError_t setup_tree_prep();
 cudaError_t launch_row_stats(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws);

@@ -107,10 +107,13 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
 
   // ---- plan the work items: every block counts all groups' items (the prefix sums below need
   //      nothing but the offsets) and writes its share of them.  An error above, or in another
-  //      block, leaves the abort flag, at which the later kernels stop.
+  //      block, stops the later kernels.  What only a sound layout can have too much of (a
+  //      group's states, the items) is left for them to report where there is no such error.
   __shared__ int s_warp[32];
   __shared__ int s_incl[kPlanThreads], s_s0[kPlanThreads], s_n[kPlanThreads];
-  int carry = 0;  // items of the groups before `base`
+  constexpr int kNone = 0x7fffffff;
+  int large = kNone;  // this thread's first group with too many states
+  int carry = 0;      // items of the groups before `base`
   // items group by group: a group's diagonal items (one per row block, block order), then
   // its off-diagonal ones; every item an off-diagonal item waits for thus comes before it
   for (int base = 0; base < sz.G; base += kPlanThreads) {
@@ -130,7 +133,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
         n = 0;
       }
       if (n > sz.maxn || n > GPO_MAX_GROUP_STATES) {
-        if (blockIdx.x == 0) report(st, GPO_ERR_UNSUPPORTED, 0, g);
+        large = min(large, g);
         n = 0;
       }
       nb = blocks_for(n);
@@ -189,9 +192,17 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
     carry += batch;
     __syncthreads();  // s_* read above
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (carry > ws.max_items) report(st, GPO_ERR_WORKSPACE, 0, carry);
-    st.p[kStItems] = carry > ws.max_items ? 0u : (uint32_t)carry;
+  if (blockIdx.x != 0) return;
+  __shared__ int s_large;
+  if (threadIdx.x == 0) s_large = kNone;
+  __syncthreads();
+  if (large != kNone) atomicMin(&s_large, large);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int code = s_large != kNone ? GPO_ERR_UNSUPPORTED : (carry > ws.max_items ? GPO_ERR_WORKSPACE : 0);
+    st.p[kStPlan] = (uint32_t)code;
+    st.p[kStPlanIndex] = (uint32_t)(code == GPO_ERR_UNSUPPORTED ? s_large : carry);
+    st.p[kStItems] = (uint32_t)(code != 0 ? kPlanFault : carry);
   }
 }
 
@@ -409,7 +420,8 @@ __global__ void __launch_bounds__(256) row_stats_kernel(gpo_batch b, Sizes sz, W
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     if (lane == 0) {
-      if (!isfinite(s2)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 1, (int)row);
+      const Status st{ws.status, ws.tag};
+      if (!isfinite(s2) && !plan_fault(st)) report(st, GPO_ERR_NONFINITE, 1, (int)row);
       ws.nrm2[row] = s2;
       ws.rn[row] = s2 > 0.f ? 1.0f / sqrtf(s2) : 0.f;
     }
@@ -492,6 +504,7 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
     v1 = max(v0, min(v1, sz.N));
   }
   const int nstate = v1 - v0, nroot = b.root_emb ? sz.g1 - sz.g0 : 0;
+  int bad = -1;  // a job with a non-finite sum
   for (int64_t jj = warp; jj < (int64_t)nstate + nroot; jj += nwarps) {
     const int64_t job = jj < nstate ? v0 + jj : sz.N + sz.g0 + (jj - nstate);
     if (job >= sz.N) {  // |prompt embedding|^2
@@ -499,7 +512,7 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
       float2 n2, dot;
       exact_pair_sums<kBf16>(b.root_emb, g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
       if (lane == 0) {
-        if (!isfinite(n2.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, (int)job);
+        if (!isfinite(n2.x)) bad = (int)job;
         ws.x_root_n2[g] = n2;
       }
       continue;
@@ -523,7 +536,7 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
     float2 n2, dot;
     exact_pair_sums<kBf16>(b.emb, (int64_t)v * sz.stride, pbase, poff, pbase != nullptr, sz.d, lane, n2, dot);
     if (lane == 0) {
-      if (!isfinite(n2.x) || !isfinite(dot.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, v);
+      if (!isfinite(n2.x) || !isfinite(dot.x)) bad = v;
       ws.x_n2[v] = n2;
       ws.x_dot[v] = dot;
       if (!kBf16) {  // the norms of the threshold test (bf16: from the similarity stage or row_stats)
@@ -532,6 +545,8 @@ __global__ void __launch_bounds__(256) exact_stats_kernel(gpo_batch b, Sizes sz,
       }
     }
   }
+  const Status st{ws.status, ws.tag};
+  if (bad >= 0 && (kBf16 || !plan_fault(st))) report(st, GPO_ERR_NONFINITE, 3, bad);  // (fp32: the kernel after prep)
 }
 
 // bf16 rows (16-byte aligned, d a multiple of 32): a warp takes 8 consecutive rows, lane
@@ -757,7 +772,7 @@ __global__ void __launch_bounds__(256) exact_stats_lane_kernel(gpo_batch b, Size
 }
 
 // |prompt embedding|^2 of groups [g0, g1), one warp each (the streamed kernel covers the states).
-__global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, Ws ws) {
+__global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, Ws ws, bool after_prep) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -765,17 +780,19 @@ __global__ void __launch_bounds__(256) root_norms_kernel(gpo_batch b, Sizes sz, 
     float2 n2, dot;
     exact_pair_sums<true>(b.root_emb, g * sz.stride, nullptr, 0, false, sz.d, lane, n2, dot);
     if (lane == 0) {
-      if (!isfinite(n2.x)) report(Status{ws.status, ws.tag}, GPO_ERR_NONFINITE, 3, (int)(sz.N + g));
+      const Status st{ws.status, ws.tag};
+      if (!isfinite(n2.x) && !(after_prep && plan_fault(st))) report(st, GPO_ERR_NONFINITE, 3, (int)(sz.N + g));
       ws.x_root_n2[g] = n2;
     }
   }
 }
 
-cudaError_t launch_root_norms(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws) {
+cudaError_t launch_root_norms(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
+                              bool after_prep) {
   int64_t blocks = ((int64_t)(sz.g1 - sz.g0) + 7) / 8;
   if (blocks < 1) return cudaSuccess;
   if (blocks > (int64_t)lc.num_sms * 8) blocks = (int64_t)lc.num_sms * 8;
-  root_norms_kernel<<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws);
+  root_norms_kernel<<<(int)blocks, 256, 0, lc.stream>>>(b, sz, ws, after_prep);
   return cudaGetLastError();
 }
 
@@ -790,7 +807,7 @@ cudaError_t launch_exact_stats(const LaunchCtx& lc, const gpo_batch& b, const Si
     const int64_t bcap = (int64_t)lc.num_sms * 32;
     blocks = blocks < 1 ? 1 : (blocks > bcap ? bcap : blocks);
     if (b.root_emb) {  // first: the norms-based path reads them
-      const cudaError_t e = launch_root_norms(lc, b, sz, ws);
+      const cudaError_t e = launch_root_norms(lc, b, sz, ws, false);
       if (e != cudaSuccess) return e;
     }
     if (with_norms)

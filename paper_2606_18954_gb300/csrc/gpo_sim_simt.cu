@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(kThreads) sim_simt_kernel(gpo_batch b, Sizes s
   const Status st{ws.status, ws.tag};
   const int it = blockIdx.x / kSubs, sub = blockIdx.x % kSubs;
   const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
+  if (nitems < 0 && blockIdx.x == 0) plan_fault(st);
   if (it >= nitems || aborted(st)) return;
   const Item item = ws.items[it];
   const GroupInfo gi = ws.groups[item.group];

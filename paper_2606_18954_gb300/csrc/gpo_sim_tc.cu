@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
-  if (aborted(st) || nitems == 0) return;  // (a CTA without items has its share of the statistics)
+  if (nitems < 0) plan_fault(st);
+  if (aborted(st) || nitems <= 0) return;  // (a CTA without items has its share of the statistics)
   const int KT = (sz.d + kTileK - 1) / kTileK;
 
   if (threadIdx.x == 0) {
