@@ -113,7 +113,9 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
   __shared__ int s_incl[kPlanThreads], s_s0[kPlanThreads], s_n[kPlanThreads];
   constexpr int kNone = 0x7fffffff;
   int large = kNone;  // this thread's first group with too many states
-  int carry = 0;      // items of the groups before `base`
+  // items of the groups before `base`: 64 bits, since offsets that do not partition the batch
+  // (reported above, or by another block) can give millions of groups the same 4096 states
+  int64_t carry = 0;
   // items group by group: a group's diagonal items (one per row block, block order), then
   // its off-diagonal ones; every item an off-diagonal item waits for thus comes before it
   for (int base = 0; base < sz.G; base += kPlanThreads) {
@@ -146,7 +148,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
       gi.n = n;
       gi.r0 = go[g];
       gi.nr = go[g + 1] - gi.r0;
-      gi.blk0 = carry + incl - cnt;
+      gi.blk0 = (int)(carry + incl - cnt);  // (read only if the total is within max_items)
       gi.nblk = nb;
       gi.off0 = gi.blk0 + nb;
       gi.noff = cnt - nb;
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
       }
       const int gn = s_n[lo], gs0 = s_s0[lo], gnb = blocks_for(gn);
       int idx = j - (lo > 0 ? s_incl[lo - 1] : 0);  // item index within the group
-      const int k = carry + j;
+      const int64_t k = carry + j;
       if (k >= ws.max_items) continue;
       Item it;
       it.group = base + lo;
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(kPlanThreads) prep_kernel(gpo_batch b, Sizes s
     const int code = s_large != kNone ? GPO_ERR_UNSUPPORTED : (carry > ws.max_items ? GPO_ERR_WORKSPACE : 0);
     st.p[kStPlan] = (uint32_t)code;
     st.p[kStPlanIndex] = (uint32_t)(code == GPO_ERR_UNSUPPORTED ? s_large : carry);
-    st.p[kStItems] = (uint32_t)(code != 0 ? kPlanFault : carry);
+    st.p[kStItems] = (uint32_t)(code != 0 ? kPlanFault : (int)carry);
   }
 }
 
