@@ -194,11 +194,12 @@ __device__ __forceinline__ void tile_links(SimtSmem& sm, const gpo_batch& b, con
 }
 
 template <bool kBf16>
-__global__ void __launch_bounds__(kThreads) sim_simt_kernel(gpo_batch b, Sizes sz, Ws ws, float kappa, int rule) {
+__global__ void __launch_bounds__(kThreads)
+    sim_simt_kernel(gpo_batch b, Sizes sz, Ws ws, float kappa, int rule, int first) {
   extern __shared__ __align__(16) unsigned char simt_smem[];
   SimtSmem& sm = *reinterpret_cast<SimtSmem*>(simt_smem);
   const Status st{ws.status, ws.tag};
-  const int it = blockIdx.x / kSubs, sub = blockIdx.x % kSubs;
+  const int it = first + (int)(blockIdx.x / kSubs), sub = blockIdx.x % kSubs;
   const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
   if (nitems < 0 && blockIdx.x == 0) plan_fault(st);
   if (it >= nitems || aborted(st)) return;
@@ -254,12 +255,23 @@ cudaError_t setup_sim_simt() {
 cudaError_t launch_sim_simt(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                             const Params& p) {
   if (ws.max_items < 1) return cudaSuccess;
-  const unsigned grid = (unsigned)ws.max_items * kSubs;  // max_items < 2^27 (layout)
-  if (b.emb_dtype == GPO_EMB_BF16)
-    sim_simt_kernel<true><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule);
-  else
-    sim_simt_kernel<false><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule);
-  return cudaGetLastError();
+  // as many launches as keep a grid's blocks within 2^31 - 1 (layout allows 2^30 items; the debug
+  // build has a limit that its tests pass)
+#ifdef GPO_DEBUG
+  constexpr int kItems = 8;
+#else
+  constexpr int kItems = 0x7fffffff / kSubs;
+#endif
+  for (int first = 0; first < ws.max_items; first += kItems) {
+    const unsigned grid = (unsigned)min(ws.max_items - first, kItems) * kSubs;
+    if (b.emb_dtype == GPO_EMB_BF16)
+      sim_simt_kernel<true><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule, first);
+    else
+      sim_simt_kernel<false><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule, first);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace gpo
