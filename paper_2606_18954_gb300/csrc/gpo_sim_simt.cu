@@ -4,7 +4,8 @@
 // accumulation.
 //
 // One CTA per 64 x 32 tile of a work item (a 128-row block against up to 256 columns: two row
-// halves by eight column chunks; tiles left of a diagonal item's diagonal are empty).  Two
+// halves by eight column chunks, fewer where no group has states for them; tiles left of a
+// diagonal item's diagonal are empty).  Two
 // parts of 64 threads, each half of every stage's k: thread (ti, tj) = (t / 8, t % 8) of a part
 // owns the outputs of rows ti + 8 a and columns tj + 8 c (a < 8, c < NC), per four elements of
 // k one 16-byte chunk of each of its 8 rows and NC columns and 32 NC fma; the second part's
@@ -33,7 +34,6 @@ constexpr int kParts = 2;              // parts: each half of every stage's k
 constexpr int kThreads = kParts * kPart;
 constexpr int kKc = 32;                // k elements of a stage
 constexpr int kLd = kKc + 4;           // row stride in shared memory (floats)
-constexpr int kSubs = 16;              // tiles of a work item: 2 row halves x 8 column chunks
 static_assert(kTileM == 2 * kTile && kTileN == 8 * kCols && kTile == 2 * kCols, "tiles of a work item");
 
 struct SimtSmem {
@@ -199,14 +199,14 @@ __global__ void __launch_bounds__(kThreads)
   extern __shared__ __align__(16) unsigned char simt_smem[];
   SimtSmem& sm = *reinterpret_cast<SimtSmem*>(simt_smem);
   const Status st{ws.status, ws.tag};
-  const int it = first + (int)(blockIdx.x / kSubs), sub = blockIdx.x % kSubs;
+  const int it = first + (int)blockIdx.z;
   const int nitems = (int)*((volatile uint32_t*)&st.p[kStItems]);
-  if (nitems < 0 && blockIdx.x == 0) plan_fault(st);
+  if (nitems < 0 && it == first) plan_fault(st);
   if (it >= nitems || aborted(st)) return;
   const Item item = ws.items[it];
   const GroupInfo gi = ws.groups[item.group];
   const int send = gi.s0 + gi.n;
-  const int row0 = item.row0 + kTile * (sub & 1), col0 = item.col0 + kCols * (sub >> 1);
+  const int row0 = item.row0 + kTile * (int)blockIdx.x, col0 = item.col0 + kCols * (int)blockIdx.y;
   const int nr = min(kTile, send - row0), nc = min(kCols, item.col0 + item.ncols - col0);
   if (nr <= 0 || nc <= 0 || col0 < row0) return;
   const bool tree = ws.tree_end != nullptr;
@@ -255,15 +255,20 @@ cudaError_t setup_sim_simt() {
 cudaError_t launch_sim_simt(const LaunchCtx& lc, const gpo_batch& b, const Sizes& sz, const Ws& ws,
                             const Params& p) {
   if (ws.max_items < 1) return cudaSuccess;
-  // as many launches as keep a grid's blocks within 2^31 - 1 (layout allows 2^30 items; the debug
-  // build has a limit that its tests pass)
+  // A block per tile that some group has states for (row halves x column chunks x items): with all
+  // 16 the blocks of the others, which end at once, were most of the time of small groups (16384
+  // branching groups of at most 6 states 817 -> 119 us, 2048 of 12 111 -> 25 us; the same as one
+  // dimension, with divisions by halves and chunks, costs 4 groups of 257 states 28.3 -> 30.3 us).
+  // As many launches as the grid's third dimension asks for (the debug build has a limit that
+  // its tests pass).
 #ifdef GPO_DEBUG
   constexpr int kItems = 8;
 #else
-  constexpr int kItems = 0x7fffffff / kSubs;
+  constexpr int kItems = 65535;
 #endif
+  const unsigned halves = sz.maxn > kTile ? 2 : 1, chunks = (unsigned)min(kTileN, sz.maxn + kCols - 1) / kCols;
   for (int first = 0; first < ws.max_items; first += kItems) {
-    const unsigned grid = (unsigned)min(ws.max_items - first, kItems) * kSubs;
+    const dim3 grid(halves, chunks, (unsigned)min(ws.max_items - first, kItems));
     if (b.emb_dtype == GPO_EMB_BF16)
       sim_simt_kernel<true><<<grid, kThreads, sizeof(SimtSmem), lc.stream>>>(b, sz, ws, (float)p.kappa, p.rule, first);
     else

@@ -49,3 +49,28 @@ def test_tile_edges(gp_mod, dtype, d, tree):
     out = gp(db, components=True, nodes=True)
     gp.check()
     compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, params), f"{dtype} d={d} tree={tree}")
+
+
+@pytest.mark.parametrize("most", [4, 33, 65])
+def test_many_small_groups(gp_mod, most):
+    """Tiles only where some group has states for them (row halves x column chunks by the declared
+    largest group), and more work items than one launch takes."""
+    G = 40000 if most == 4 else 300
+    rng = np.random.default_rng(most)
+    n = rng.integers(1, 3, 2 * G)  # two rollouts per group
+    n[:2] = [1, most - 1]
+    so = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+    N = int(so[-1])
+    emb = np.zeros((N, 8), np.float32)
+    emb[np.arange(N), rng.integers(0, 8, N)] = rng.uniform(0.5, 2.0, N).astype(np.float32)  # cosines 0 or 1
+    lens = rng.integers(1, 4, N).astype(np.int32)
+    to = np.concatenate([[0], np.cumsum(lens)])[so].astype(np.int64)
+    b = dict(group_rollout_off=(2 * np.arange(G + 1)).astype(np.int32), rollout_step_off=so, step_len=lens,
+             rollout_token_off=to, emb=emb, emb_dtype="f32", reward=rng.integers(0, 2, 2 * G).astype(np.uint8),
+             kappa=0.9, w=0.7, lambda_eff=1.0)
+    gp = gp_mod.GraphPO(kappa=0.9, w=0.7, lambda_eff=1.0, flags=gp_mod.binding.FLAG_TILED)
+    db = gp_mod.Batch.from_arrays(b, device="cuda")
+    assert db.max_states_per_group == most
+    out = gp(db, components=True, nodes=True)
+    gp.check()
+    compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, oracle_params(b)), f"{most}")
