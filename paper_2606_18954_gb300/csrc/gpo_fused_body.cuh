@@ -16,8 +16,14 @@ constexpr int kReps = kEpiThreads / 128;        // drain warps per accumulator l
 constexpr int kWarpEdges = 256;                 // linked pairs listed per epilogue warp and group
 constexpr int kEdgeList = kWarpEdges * (kEpiThreads / 32);
 // Groups of two passes wait for the second one's MMAs after draining the first: the token scatter
-// of the group before is put there (deferred_tokens).
+// of the group before is put there (deferred_tokens) where that wait is longer than the scatter.
+// Not before a group of one pass, or with narrow rows: the scatter by the drain warps alone then
+// only delays the drain.  Put off / at once, us: 512 groups of 370 states (nearly all of two
+// passes) d = 64 141 / 135, 256 169 / 165, 384 183 / 180, 512 193 / 194, 768 233 / 238, 1024
+// 253 / 262, 2048 403 / 413; 512 of 320 d = 512 169 / 171, 1024 219 / 228; 512 of 256 states
+// (one pass, put off whatever follows) d = 1024 173 / 168, 512 branching ones of 200 222 / 217.
 constexpr bool kDeferTokens = kMaxN > 2 * kTileM;
+constexpr int kDeferD = 512;                    // narrowest rows for which the scatter is put off
 constexpr int kBarGroup = 1;                    // named barrier of the group warps
 constexpr int kBarEpi = 2;                      // named barrier of the drain warps
 constexpr int kBarSetup = 3;                    // named barrier of warps 2 and 3 (early set-up)
@@ -137,6 +143,7 @@ struct __align__(16) GroupSmem {
   int overflow;          // some warp found more pairs than its part of elist holds
   int nstat[2];          // group_eta_stats: rows with a dot, rows with the norm alone (group_row_stats:
                          // the next block of 8 rows)
+  bool wait_ahead;       // the CTA's next group has two passes
   int put_off;           // scatter put off: states of the group, its first token,
   int64_t dbase;
   uint32_t dts[kDeferTokens ? kMaxN + 1 : 1];  // of each state relative to it (they follow one another),
@@ -735,6 +742,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
         }
       }
 
+      if (kDeferTokens && gt == 0) {  // (read after the drain)
+        int r2, nr2, s2, n2;
+        gs->wait_ahead = sz.d >= kDeferD && g + (int64_t)gridDim.x < sz.g1 &&
+                         group_active(b, sz, g + (int)gridDim.x, r2, nr2, s2, n2) && plan_passes(n2) == 2;
+      }
+
       // ---- drain the accumulator pass by pass (warps 4..15)
       bool fail = false;
       if (epi) {
@@ -969,22 +982,18 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
                            o.group_eff ? o.group_eff + g : nullptr, o.group_eff_graph ? o.group_eff_graph + g : nullptr);
         }
         // ---- every token of an edge carries the edge's advantage (Sec. 4.5), state-major, a
-        //      half-warp per state.  With a group to follow on this CTA it is put off to that
-        //      group's last wait for its MMAs: a group of two passes waits ~13 us for the second one
+        //      half-warp per state.  With a group of two passes to follow on this CTA it is put off
+        //      to that group's last wait for its MMAs: it waits ~13 us for the second one
         //      (320 states of 2 KB), the scatter is ~6.5 us of stores, and the next group starts that
-        //      much earlier (512 groups of 320 states 241 -> 231 us).  The drain warps do it: with
+        //      much earlier (kDeferD).  The drain warps do it: with
         //      warps 2 and 3 as well, a second copy of the code, 128 groups of 256 states lose more
         //      (51.3 -> 52.0) than these gain, and those two alone take longer than the wait (268).
         //      Only in the instance whose groups can take two passes; the per-token components
         //      go out at once.  Streaming stores: they take no place in L2 from the rows that are
         //      still to be read (256 groups of 56 states with every output 53.4 -> 49.8 us).
         const bool more = o.adv_cor || o.adv_eff || o.eff_mask;
-        bool later = false;
-        if (kDeferTokens && !more && g + (int64_t)gridDim.x < sz.g1) {
-          int r2, nr2, s2, n2;
-          later = group_active(b, sz, g + (int)gridDim.x, r2, nr2, s2, n2) &&
-                  gs->tstart[n - 1] + gs->slen[n - 1] - gs->tstart[0] <= 0xFFFFFFFFll;
-        }
+        const bool later = kDeferTokens && !more && gs->wait_ahead &&
+                           gs->tstart[n - 1] + gs->slen[n - 1] - gs->tstart[0] <= 0xFFFFFFFFll;
         if (later) {
           const int64_t base = gs->tstart[0];
           if (gt == 0) {

@@ -34,3 +34,19 @@ def test_deferred_scatter(gp_mod, kind, steps, tokens, components):
     out = gp(db, components=components, nodes=True)
     gp.check()
     compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, params), f"{kind} {steps}")
+
+
+@pytest.mark.parametrize("d", [504, 512])
+def test_deferred_before_two_passes(gp_mod, d):
+    """Put off only before a group of two passes (289 to 384 states) and with rows of at least 512:
+    groups of one and of two passes in turn on every CTA that has several."""
+    spec = dataclasses.replace(W.CONFIGS["math"], groups=340, rollouts=16, d=d, centroids=24, sigma=0.05, kappa=0.9,
+                               steps=("uniform", 15, 22), lengths=("per_step", 1, 60))
+    b = dict(W.make_batch(spec, seed=6))
+    n = np.diff(np.asarray(b["rollout_step_off"])[np.asarray(b["group_rollout_off"])])
+    assert (n > 288).any() and (n <= 288).any() and n.max() <= 384
+    params = oracle_params(b)
+    gp = gp_mod.GraphPO(kappa=params["kappa"], w=params["w"], lambda_eff=params["lambda_eff"])
+    out = gp(gp_mod.Batch.from_arrays(b, device="cuda"), nodes=True)
+    gp.check()
+    compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, params), f"d={d}")
