@@ -140,7 +140,10 @@ __device__ __forceinline__ bool aborted(const Status& st) {
   return is_error(*reinterpret_cast<volatile const uint64_t*>(st.p + kStError), status_tag(st));
 }
 
-__device__ __forceinline__ void report(const Status& st, int code, int where, int detail) {
+#ifndef GPO_REPORT
+#define GPO_REPORT __forceinline__
+#endif
+static __device__ GPO_REPORT void report(const Status st, int code, int where, int detail) {
   unsigned long long* w = reinterpret_cast<unsigned long long*>(st.p + kStError);
   const unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(w), t = status_tag(st);
   if (is_error(old, t)) return;  // not the first error
