@@ -323,6 +323,34 @@ uint64_t fresh_tag() {
   }
 }
 
+// Fused path: whether the compensated statistics of the groups after each CTA's first come from a
+// launch on the whole GPU first (exact_stats, every row) or from the kernel, once a group's
+// classes are known (group_eta_stats, the rows that need them): a serial step of about the same
+// time for any group, so small groups, many of them per CTA and branching ones (which need 0.85
+// of their rows) prefer the launch, wide rows the kernel.  Launch / kernel, us, d a multiple of
+// 32 (the launch takes eight rows per warp):
+//   groups x states    d = 64       256        384        512        768        896        1024
+//   512 x 320       123 / 137  152 / 153  169 / 160  182 / 167  212 / 200  229 / 215  244 / 219
+//   512 x 256        98 / 106  121 / 118  134 / 123  146 / 130  167 / 150  179 / 159  188 / 167
+//   1024 x 112       76 / 83    92 / 91   103 / 98   113 / 101  129 / 116  137 / 122  153 / 129
+//   2048 x 112      141 / 160  168 / 174  185 / 184  202 / 189  235 / 217  251 / 225  271 / 236
+//   4096 x 56       203 / 237  233 / 261  250 / 267  269 / 273  302 / 300  318 / 307  341 / 314
+//   4096 x 24       151 / 200  167 / 209  178 / 217  189 / 224  206 / 236  215 / 238  237 / 246
+//   512 x 56         35 / 35    39 / 37    43 / 39    47 / 41    58 / 48    61 / 50    64 / 49
+//   512 branching   124 / 153  141 / 160  152 / 168  167 / 171  189 / 197  192 / 205  219 / 214
+//   200 branching    65 / 74    71 / 79    80 / 85    88 / 90    99 / 106  101 / 107  107 / 108
+// Other widths take the launch's one row per warp: 512 x 320, d = 72 181 / 136, 248 197 / 151,
+// 520 251 / 194; 512 branching d = 72 152 / 154, 248 161 / 160, 392 183 / 169, 200 branching
+// d = 72 69 / 75.
+bool rest_stats_first(const gpo_batch& b, const Sizes& sz, int grid) {
+  const int64_t groups = (int64_t)sz.g1 - sz.g0;
+  if (groups <= grid) return false;
+  const bool eight_rows = sz.d % 32 == 0;
+  if (b.parent) return sz.d <= 256 || (eight_rows && sz.d < 1024);
+  return eight_rows && (sz.d <= 256 || (sz.d <= 1024 && groups >= 4 * (int64_t)grid &&
+                                        (int64_t)sz.N * sz.d < (int64_t)40960 * sz.G));
+}
+
 // Next-layer budget request of gpo_layer_budget (mode 1 of the kernels).
 struct BudgetReq {
   int layer, b_next;
@@ -454,11 +482,8 @@ gpo_status compute_impl(gpo_ctx* ctx, const gpo_batch* batch, const gpo_outputs*
   } else if (fused32) {
     if (e == cudaSuccess) e = stage("fused_f32", [&] { return launch_fused_f32(lc, b, *out, sz, ws, pp); });
   } else if (fused) {
-    // rows of d <= kRestStatsD: the statistics of the groups after each CTA's first by a launch
-    // on the whole GPU first, a few us that group_eta_stats' steps would cost every group (512
-    // groups of 320 states: d = 64 138 against 151 us, 256 162 / 167, 512 201 / 189, 1024 277 / 257)
     const int grid = fused_grid(lc, sz);
-    if (e == cudaSuccess && !bud && sz.d <= kRestStatsD && g1 - g0 > (int64_t)grid) {
+    if (e == cudaSuccess && !bud && rest_stats_first(b, sz, grid)) {
       pp.rest_stats = 1;
       Sizes rest = sz;
       rest.g0 = sz.g0 + grid;
