@@ -209,10 +209,10 @@ def _raw_stream(stream, dev) -> ctypes.c_void_p:
     import torch
     if stream is not None:
         return ctypes.c_void_p(stream.cuda_stream)
-    if dev.type != "cuda":
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # a private name of torch's, where it has it:
+    if raw is None or dev.type != "cuda":                       # current_stream() builds an object, 2 us
         return ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
-    index = torch.cuda.current_device() if dev.index is None else dev.index
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(index))  # current_stream() builds an object: 2 us
+    return ctypes.c_void_p(raw(torch.cuda.current_device() if dev.index is None else dev.index))
 
 
 @dataclasses.dataclass
