@@ -110,8 +110,8 @@ def algorithmic(b):
     path_bytes = zb + 4 * N + meta + R + 4 * T
     # exact_stats: per embedding element two exact products (|z|^2 and the parent dot) and two
     # compensated additions (TwoSum: 6 operations plus the error accumulation): 16 fp32 operations,
-    # the figure the notes are held to; the kernels spend 8 (biased sums), and the group-resident
-    # ones only on the rows whose eta can reach a result
+    # the figure the notes are held to (8 where the norms give the sums a bias); the bf16
+    # group-resident kernel sums only the rows whose eta can reach a result (alu_note)
     alu_x = 16.0 * N * d
     stages = {
         "exact_stats": (zb + 16 * N, 0.0, alu_x),
@@ -467,9 +467,11 @@ def kernel_roofline(name, stage_ms, alg, hbm, tc, workload):
 
 def alu_note(name, stage_ms, alg):
     """The compensated statistics' fp32 operations of a kernel against the fp32 issue peak
-    (an implementation device for the accuracy of eta, not part of the roofline)."""
+    (an implementation device for the accuracy of eta, not part of the roofline).  None for the
+    bf16 group-resident kernel: it sums 0.2 to 0.85 of the rows, which ones the classes decide,
+    so the operations of all rows over its time would be a rate of work that is not done."""
     st = alg["stages"][name]
-    if len(st) < 3 or not st[2]:
+    if len(st) < 3 or not st[2] or name == "fused":
         return None
     peak = alu_peak_tops()
     achieved = st[2] / (stage_ms[name] / 1e3) / 1e12

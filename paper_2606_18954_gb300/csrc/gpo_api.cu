@@ -1,7 +1,7 @@
 // Host implementation of the C ABI declared in include/graphpo.h: argument
 // checks, workspace layout, TMA descriptor encoding and the launch sequence
-//   fused (the group-resident kernels; for rows of d <= 256 and more groups than CTAs the
-//   compensated statistics of the later groups first), or
+//   fused (the group-resident kernels; with several groups per CTA, where that is faster, the
+//   compensated statistics of the later groups first: rest_stats_first), or
 //   prep (validate + plan) -> row statistics (CUDA-core similarity only) -> similarity merge
 //   (on the tensor cores with the compensated statistics) -> per-group advantages -> per-token
 //   scatter

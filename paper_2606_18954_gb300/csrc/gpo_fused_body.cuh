@@ -213,8 +213,8 @@ __device__ __forceinline__ float pick(const uint32_t (&r)[32], int j) {
 // and dependent sums at 14 warps per SM (a third of the issue slots used).  Results as float
 // pairs: |z|^2 in (rn, thr), free once the pairs are tested, the dot in (ecor, eeff).
 // Whole call, against the statistics of all rows (a CTA's first group while it streams in,
-// the groups after it in a launch of their own before): 512 groups of 320 states 273 -> 245 us
-// (223 with the steps since).
+// the groups after it in a launch of their own before): 512 groups of 320 states 244 -> 219 us
+// (other shapes at rest_stats_first in gpo_api.cu).
 template <class Par>
 __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes& sz, const Ws& ws, GroupSmem* gs,
                                                 int g, int s0, int n, bool need, Par par, int gt, int wg, int lane,
@@ -276,11 +276,15 @@ __device__ __forceinline__ void group_eta_stats(const gpo_batch& b, const Sizes&
 // first group, when they would otherwise wait for the stream, of a branching batch or with
 // rows of d < kEarlyD.  All rows' statistics then take no longer than the stream and what
 // follows it, while group_eta_stats is a serial step after the classes; with wider rows its
-// third of a chain batch's rows is the less (128 groups of 256 states, us, these statistics
-// against group_eta_stats: d = 64 31.4 / 39.6, 256 37.9 / 43.6, 512 43.7 / 45.8, 768 60.0 /
-// 60.1, 1024 60.0 / 58.0, 2048 111 / 95; 256 groups of 56: d = 256 27.2 / 33.4, 768 34.4 / 37.5,
-// 1024 39.5 / 39.6, 2048 58.0 / 51.9).  A branching batch reads 0.85 of its eta's (tree, d =
-// 1024: 71.0 / 74.4).  The calling warps claim blocks of 8 rows from gs->nstat[0] until none is
+// third of a chain batch's rows is the less.  These statistics / group_eta_stats, us a call:
+//   groups x states   d = 64    256       512       768       896       1024      1280      1536      2048
+//   128 x 256         27 / 35   31 / 37   39 / 41   45 / 50   49 / 52   52 / 53   60 / 61   68 / 65   103 / 87
+//   128 x 340         33 / 43   39 / 45   52 / 51   63 / 65   69 / 68   77 / 71   90 / 83   102 / 91  128 / 112
+//   256 x 56          19 / 24   21 / 25   25 / 26   29 / 29   31 / 30   33 / 32   38 / 37   41 / 38   50 / 45
+//   256 x 112         23 / 31   27 / 31   33 / 33   40 / 40   43 / 42   46 / 42   53 / 49   59 / 52   73 / 62
+//   16 x 56           19 / 23   20 / 23   21 / 24   23 / 26   25 / 27   25 / 28   28 / 31   31 / 34   36 / 40
+// A branching batch reads 0.85 of its eta's: 128 groups of 200 d = 64 40 / 52, 1024 67 / 74, 2048
+// 94 / 103.  The calling warps claim blocks of 8 rows from gs->nstat[0] until none is
 // left, so that warps that join late or run slower take fewer (eight_rows_sums).  Parents: with `early` (chain
 // layout, before the group's set-up) the previous state for every state but the group's first
 // (the set-up fixes the rollouts' first states afterwards: their parent is the prompt root);
@@ -668,7 +672,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       const bool stats_here = p.mode == 0 && (tree || sz.d < kEarlyD) && first;
       const bool early = stats_here && !tree && b.root_emb == nullptr;
       if (early && epi) group_row_stats(b, sz, ws, gs, g, s0, n, false, true, lane, st);
-
 
       if (tree) {
         tree_setup(b, sz, gs, g, r0, nr, s0, n, gt, wg, lane, st);

@@ -14,11 +14,12 @@
 //             per token the ratio, the clipped surrogate, the k3 KL estimate, the gradient
 //             (one 16-byte store per chunk); sums in fp32 per tile, float pairs across tiles,
 //             per-CTA partials combined by the last CTA in a fixed order (deterministic).
-// 12 bytes per token (16 with the KL term) plus ~16 bytes per edge; bound by issue (57 % of the
+// 12 bytes per token (16 with the KL term) plus ~16 bytes per edge; bound by issue (58 % of the
 // slots) and by the latency of a tile's loads.  While a warp waits for its tokens or edges
 // the SM's others compute, which CTA-wide steps of 4096 tokens with three barriers each did
-// not allow: 38.3 M tokens in the split form with the KL term 183 -> 128 us (4.8 TB/s), 4.7 M
-// in the dual form 27.3 -> 23.2 us.  Tiles of 256 tokens: 132 / 25.2 us.
+// not allow: 38.3 M tokens in the split form with the KL term 175 -> 118 us (5.2 TB/s), 4.7 M
+// in the dual form 19.1 -> 17.0, 512 groups of edges of 1 to 3 tokens 32 -> 11 us (calls one
+// after another, captured).  Tiles of 256 tokens cost 3 % (split) and 9 % (dual) more.
 #include "gpo_internal.cuh"
 
 namespace gpo {

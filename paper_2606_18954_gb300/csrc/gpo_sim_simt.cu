@@ -17,9 +17,9 @@
 // a tile are united in shared memory, then one union per non-root state in the batch's label
 // forest (ws.lab).
 //
-// Bound by fp32 issue (64 % of the slots while an SM has work, three quarters of them fma):
-// 64 groups of 257 states, d = 1024 take 184 us, of which the fma of their upper-triangle
-// tiles are 78 us of the fp32 pipe.  Before, one CTA of 256 threads per item with scalar loads
+// Bound by issue (69 % of the slots while an SM has work, 65 % of the instructions fma):
+// 64 groups of 257 states, d = 1024 take 184 us, of which the 2.83 G fma of their upper-triangle
+// tiles are 70 us of the fp32 pipe at 2070 MHz.  Before, one CTA of 256 threads per item with scalar loads
 // transposed into shared memory: 795 us.  The same tile with 64 threads and whole k, one wave
 // of long CTAs: 238 us; with four parts 205 us; packed f32x2 fma 256 us.
 #include "gpo_internal.cuh"

@@ -78,7 +78,7 @@ __device__ __forceinline__ void epi_sync() {
 // Bits a..31 of a word (all for a <= 0, none for a >= 32).
 __device__ __forceinline__ uint32_t bits_from(int a) { return a <= 0 ? 0xFFFFFFFFu : (a >= 32 ? 0u : 0xFFFFFFFFu << a); }
 
-// Barrier of the 4 epilogue warps that also ORs a flag across them, so that
+// Barrier of the epilogue warps that also ORs a flag across them, so that
 // they all take the same early exit.
 __device__ __forceinline__ bool epi_any(bool flag) {
   uint32_t out;
@@ -348,8 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t r[32];
         tmem_ld_32x32b_x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * kTileN + ch * 32), r);
         tmem_wait_ld();
-        // <z of the block's last row, z of the next block's first row>: the parent dot of
-        // the next block's first state when it continues the same rollout
+        // bit j of `miss` = sign of acc_j / |z_j| - kappa |z_i| (one fma): set below the threshold
         uint32_t mp[4] = {0u, 0u, 0u, 0u};
         const float4* rn4 = reinterpret_cast<const float4*>(ctl->cm_rn + ch * 32);
 #pragma unroll

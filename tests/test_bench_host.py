@@ -100,5 +100,12 @@ def test_kernel_roofline_takes_the_slower_of_bytes_and_flops():
     assert bench.alu_note("similarity", ms, a) is None
 
 
+def test_no_rate_of_sums_that_are_skipped():
+    """The bf16 group-resident kernel sums only the rows whose eta can reach a result."""
+    a = bench.algorithmic(W.make_batch(W.CONFIGS["math"].scaled(groups=2)))
+    assert bench.alu_note("fused", {"fused": 0.05}, a) is None
+    assert bench.alu_note("fused_f32", {"fused_f32": 0.05}, a)["fp32_ops"] == a["stages"]["fused_f32"][2]
+
+
 def test_whole_job_value():
     assert bench.whole_job_value(4_000_000, 2.0) == pytest.approx(2e9)
