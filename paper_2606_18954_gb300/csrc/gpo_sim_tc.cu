@@ -38,6 +38,8 @@
 //                      157 us after it (two such warps 840 us, ten 414; TwoSum, which needs no
 //                      norms, 451)
 // The Gram block Z_g Z_g^T is never written to memory.
+// Error reports out of line, as in the fused kernels: inlined they cost spills.
+#define GPO_REPORT __noinline__
 #include "gpo_internal.cuh"
 
 namespace gpo {
