@@ -17,6 +17,8 @@
 // Replaces the tiled path's six launches for such batches (prep, row norms, similarity,
 // statistics, per-group math, tokens).  Groups of at most 64 states run with 512 threads
 // (the Gram's k range split between the block's halves), larger ones with 256.
+// Error reports out of line (300 groups of 60 states, d = 128: 56.8 -> 55.6 us).
+#define GPO_REPORT __noinline__
 #include "gpo_group_math.cuh"
 
 namespace gpo {
