@@ -36,17 +36,23 @@ def test_deferred_scatter(gp_mod, kind, steps, tokens, components):
     compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, params), f"{kind} {steps}")
 
 
+@pytest.mark.parametrize("tree", [False, True])
 @pytest.mark.parametrize("d", [504, 512])
-def test_deferred_before_two_passes(gp_mod, d):
+def test_deferred_before_two_passes(gp_mod, d, tree):
     """Put off only before a group of two passes (289 to 384 states) and with rows of at least 512:
     groups of one and of two passes in turn on every CTA that has several."""
-    spec = dataclasses.replace(W.CONFIGS["math"], groups=340, rollouts=16, d=d, centroids=24, sigma=0.05, kappa=0.9,
-                               steps=("uniform", 15, 22), lengths=("per_step", 1, 60))
-    b = dict(W.make_batch(spec, seed=6))
-    n = np.diff(np.asarray(b["rollout_step_off"])[np.asarray(b["group_rollout_off"])])
+    if tree:
+        spec = W.TreeSpec("defer", 340, (4, 5, 4, 3), d, "bf16", 24, 0.05, 0.9, ("per_step", 1, 60), ("beta", 2.0, 2.0))
+        b = dict(W.make_tree_batch(spec, seed=6))
+        n = np.diff(b["group_state_off"])
+    else:
+        spec = dataclasses.replace(W.CONFIGS["math"], groups=340, rollouts=16, d=d, centroids=24, sigma=0.05, kappa=0.9,
+                                   steps=("uniform", 15, 22), lengths=("per_step", 1, 60))
+        b = dict(W.make_batch(spec, seed=6))
+        n = np.diff(np.asarray(b["rollout_step_off"])[np.asarray(b["group_rollout_off"])])
     assert (n > 288).any() and (n <= 288).any() and n.max() <= 384
     params = oracle_params(b)
     gp = gp_mod.GraphPO(kappa=params["kappa"], w=params["w"], lambda_eff=params["lambda_eff"])
     out = gp(gp_mod.Batch.from_arrays(b, device="cuda"), nodes=True)
     gp.check()
-    compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, params), f"d={d}")
+    compare({k: v.cpu().numpy() for k, v in out.items()}, oracle_run(b, params), f"d={d} tree={tree}")
